@@ -278,21 +278,50 @@ std::string pmul(bool ps, const std::string& a, const std::string& b) {
 // The frequency loop's products (1/D = D r, the trie's complex products, Z, the sums' first terms)
 // run on the integer pipes with imul, for every table: with 32 frequencies the 85 order-2..5
 // diagrams went from 2.668 to 2.255 s once the large tables (which had kept them on the FP64 unit
-// while their kernels waited on instruction fetch) took them too.  $TAMI_JIT_INTARITH=0 keeps them
-// on the FP64 unit.
+// while their kernels waited on instruction fetch) took them too.  Where the loop has few sums the
+// integer pipes would become the bottleneck, and loop_share leaves some products on the FP64 unit.
+// $TAMI_JIT_INTARITH=0 keeps them all there.
 bool int_products(const TableHeader& h) {
   (void)h;
   const char* e = std::getenv("TAMI_JIT_INTARITH");
   return !(e && !std::strcmp(e, "0"));
 }
 
-void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero) {
+int count_of(const std::string& s, const char* what) {
+  int n = 0;
+  for (size_t at = s.find(what); at != std::string::npos; at = s.find(what, at + 1)) ++n;
+  return n;
+}
+
+// The share of a loop's products that goes to the integer pipes, so that these and the FP64 unit
+// finish together: with `loop` the generated loop whose products are all imul, and times in FP64
+// instructions (67 clocks of an SM quarter each), a product costs the integer pipes 1.1, a
+// reciprocal 0.95 and the loop's own indexing, loads and stores about 1 (measured one by one:
+// imul 74 clocks, rcp 63).  Loops with many sums keep every product on the integer pipes; the
+// evaluation example's (one denominator, no sums) moves three of its four back: 1.155 -> 0.872 ms
+// for 10^6 rows and 100 frequencies, two external frequencies (400 000 rows) 5.13 -> 4.79 ms.
+double loop_share(const std::string& loop) {
+  const double fp = count_of(loop, "fma(") + count_of(loop, " += ");
+  const double ints = 0.95 * count_of(loop, "rcp(") + 1.0;
+  const double products = count_of(loop, "imul("), cost = 1.1;
+  if (products <= 0.0) return 1.0;
+  const double on_fp = (ints + cost * products - fp) / (1.0 + cost);
+  return std::min(1.0, std::max(0.0, 1.0 - on_fp / products));
+}
+
+// share: the part of the products, spread evenly over the loop, that is written as imul
+void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
   const TableHeader& h = t.h;
   const bool ia = int_products(h);
   const bool ps = ps_products(h) && kind != kKindEnergy;
   auto PM = [&](const std::string& a, const std::string& b) { return pmul(ps, a, b); };
+  double due = 0.0;
   auto MUL = [&](const std::string& a, const std::string& b) {
-    return ia ? "imul(" + a + ", " + b + ")" : PM(a, b);
+    if (!ia) return PM(a, b);
+    due += share;
+    if (due < 1.0 - 1e-9) return a + " * " + b;
+    due -= 1.0;
+    return "imul(" + a + ", " + b + ")";
   };
   auto NEG = [&](const std::string& a) {   // sign flip (no arithmetic)
     return "__longlong_as_double(__double_as_longlong(" + a + ") ^ (long long)0x8000000000000000ull)";
@@ -729,10 +758,15 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     for (int c = 0; c < h.n_cden; ++c) o("    jsv[%d * %d + tid] = b%d;", n_sv - h.n_cden + c, B, c);
   }
   const size_t loop0 = o.s.size();
+  auto loop = [&](bool xr_zero) {
+    Out whole;
+    emit_phase2(whole, t, kind, xr_zero, 1.0);
+    emit_phase2(o, t, kind, xr_zero, loop_share(whole.s));
+  };
   o("    if (xr_zero) {");
-  emit_phase2(o, t, kind, true);
+  loop(true);
   o("    } else {");
-  emit_phase2(o, t, kind, false);
+  loop(false);
   o("    }");
   if (sv) {
     std::string loop = o.s.substr(loop0);

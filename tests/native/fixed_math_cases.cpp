@@ -1,0 +1,79 @@
+// The kernels' fixed-point reciprocal, exponential and cos/sin (csrc/tami_devmath.cuh) compiled for
+// the host and compared with long double, at the places where they can go wrong: the ends of the
+// binades and of the tables, arguments next to table points and quadrant boundaries, tiny and huge
+// arguments, zeros, infinities and NaNs.  The hardware's reciprocal estimate is replaced by a
+// rounded division that is off by RCP_OFF units in the last place.
+#include <algorithm>
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <limits>
+#include <random>
+using std::max;
+using std::min;
+#define __device__
+#define __forceinline__ inline
+#define __noinline__
+#define __align__(n) __attribute__((aligned(n)))
+struct ulonglong2 { unsigned long long x, y; };
+typedef unsigned long long u64;
+template <class A, class B> static A bits_as(B b) { A a; std::memcpy(&a, &b, sizeof a); return a; }
+static unsigned __umulhi(unsigned a, unsigned b) { return (unsigned)(((u64)a * b) >> 32); }
+static float __uint_as_float(unsigned u) { return bits_as<float>(u); }
+static unsigned __float_as_uint(float f) { return bits_as<unsigned>(f); }
+static int __float_as_int(float f) { return bits_as<int>(f); }
+static long long __double_as_longlong(double d) { return bits_as<long long>(d); }
+static double __longlong_as_double(long long d) { return bits_as<double>(d); }
+static int __double2hiint(double d) { return (int)(bits_as<u64>(d) >> 32); }
+static int __double2loint(double d) { return (int)bits_as<u64>(d); }
+static double __hiloint2double(int h, int l) { return bits_as<double>(((u64)(unsigned)h << 32) | (unsigned)l); }
+static int __clz(int x) { return x ? __builtin_clz((unsigned)x) : 32; }
+static int __clzll(long long x) { return x ? __builtin_clzll((u64)x) : 64; }
+static unsigned __funnelshift_l(unsigned lo, unsigned hi, unsigned s) { return s ? (hi << s) | (lo >> (32 - s)) : hi; }
+template <class T> static T __ldg(const T* p) { return *p; }
+static double __dmul_rn(double a, double b) { return a * b; }
+static double __dadd_rn(double a, double b) { return a + b; }
+static double __ull2double_rn(u64 a) { return (double)a; }
+static int RCP_OFF = 0;
+static float host_rcp_estimate(float x) { return __uint_as_float(__float_as_uint((float)(1.0 / (double)x)) + (unsigned)RCP_OFF); }
+using std::fabs; using std::fma; using std::fmaf; using std::fmax; using std::fmaxf; using std::fmod; using std::rint;
+#include "devmath_host.h"
+
+using namespace tami::dev;
+typedef long double L;
+static double ulp(double v) { return std::ldexp(1.0, std::ilogb(v) - 52); }
+static int failures = 0;
+static void check(bool ok, const char* what, double at, double got) {
+  if (!ok && failures++ < 20) std::printf("%s at %a: %a\n", what, at, got);
+}
+
+static std::mt19937_64 R(7);
+static double uniform(double a, double b) { return a + (b - a) * ((R() >> 11) * 0x1p-53); }
+
+static void test_rcp() {
+  const double inf = std::numeric_limits<double>::infinity();
+  for (RCP_OFF = -1; RCP_OFF <= 1; ++RCP_OFF) {
+    auto one = [](double d) {
+      const double r = rcp(d);
+      const L e = ((L)r * d - 1.0L) / d;                 // r - 1/d, the product exact to 2^-63
+      check(std::fabs((double)(e / (L)ulp(r))) <= 0.502, "rcp", d, r);
+    };
+    for (int i = 0; i < 200000; ++i) {
+      one(1.0 + i * 0x1p-52);
+      one(2.0 - (i + 1) * 0x1p-53 * 2);
+      one(std::ldexp(uniform(1, 2), (int)(R() % 2000) - 1000) * (i & 1 ? -1 : 1));
+      one(1.0 + (i & 0x7FFFFF) * 0x1p-23 + (R() & 3) * 0x1p-52);   // next to the estimate's 24 bits
+    }
+    check(rcp(1.0) == 1.0 && rcp(-4.0) == -0.25 && rcp(0x1p-1022) == 0x1p1022, "rcp exact", 1.0, rcp(1.0));
+    for (double d : {0.0, -0.0, 1e-310, inf, -inf, std::nan("")}) check(std::isnan(rcp(d)), "rcp odd", d, rcp(d));
+    check(rcp(0x1.8p1022) == 0.0 && std::signbit(rcp(-0x1p1023)), "rcp of a huge value", 0x1.8p1022, rcp(0x1.8p1022));
+  }
+  RCP_OFF = 0;
+}
+
+int main(int argc, char** argv) {
+  const char* what = argc > 1 ? argv[1] : "";
+  if (!std::strcmp(what, "rcp")) test_rcp();
+  std::printf("%d failures\n", failures);
+  return failures != 0;
+}
