@@ -71,9 +71,32 @@ static void test_rcp() {
   RCP_OFF = 0;
 }
 
+static void test_exp() {
+  const double inf = std::numeric_limits<double>::infinity(), step = std::log(2.0) / 1024;
+  auto one = [](double t) {
+    double em, unused;
+    const double y = exp_neg<true>(t, em), y0 = exp_neg<false>(t, unused);
+    check(__double_as_longlong(y) == __double_as_longlong(y0), "exp without e^t - 1", t, y0);
+    if (t > -707.0) check(std::fabs((double)(((L)y - std::exp((L)t)) / (L)ulp(y))) <= 0.51, "exp", t, y);
+    if (t < -1e-300) check(std::fabs((double)(((L)em - std::expm1((L)t)) / (L)ulp(em))) <= 0.75, "expm1", t, em);
+  };
+  for (int i = 0; i < 100000; ++i) {
+    one(-uniform(0, 1)); one(-uniform(0, 50)); one(-uniform(0, 707)); one(-uniform(0, 4 * step));
+    one(-std::pow(10.0, uniform(-299, 2.8)));
+    one(-(i % 1030000 / 1.0) * step); one(-i * step * (1 + 0x1p-52)); one(-i * step * (1 - 0x1p-53));
+  }
+  double em;
+  check(exp_neg<true>(0.0, em) == 1.0 && em == 0.0, "exp(0)", 0.0, em);
+  check(exp_neg<true>(-1e-320, em) == 1.0 && em == -1e-320, "exp(subnormal)", -1e-320, em);
+  for (double t : {-709.0, -745.2, -1023.9, -1024.0, -1e300, -inf})   // below the normal range: 0
+    check(exp_neg<true>(t, em) == 0.0 && em == -1.0, "exp underflow", t, em);
+  check(std::isnan(exp_neg<true>(std::nan(""), em)) && std::isnan(em), "exp(NaN)", 0.0, em);
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "rcp")) test_rcp();
+  if (!std::strcmp(what, "exp")) test_exp();
   std::printf("%d failures\n", failures);
   return failures != 0;
 }
