@@ -93,10 +93,43 @@ static void test_exp() {
   check(std::isnan(exp_neg<true>(std::nan(""), em)) && std::isnan(em), "exp(NaN)", 0.0, em);
 }
 
+static void test_trig() {
+  const double inf = std::numeric_limits<double>::infinity();
+  auto one = [](double k) {
+    double s, c;
+    cw_sincos(k, s, c);
+    check(std::fabs((double)((L)c - std::cos((L)k))) <= 8e-17, "cos", k, c);
+    check(std::fabs((double)((L)s - std::sin((L)k))) <= 8e-17, "sin", k, s);
+    check(cw_cos(k) == c, "cos alone", k, c);
+  };
+  for (int i = 0; i < 100000; ++i) {
+    one(uniform(-22, 22)); one(uniform(-31.9, 31.9)); one(std::pow(10.0, uniform(-300, 1.5)));
+    const double a = (i % 20000 - 10000) * (M_PI / 1024);                 // table points and the middles between
+    one(a); one(a * (1 + 0x1p-52)); one(a + uniform(-1e-9, 1e-9));
+    const double kx = uniform(-22, 22), ky = uniform(-22, 22);
+    double gx, gy;
+    const double E = line_energy(kx, ky, 1.0, -0.3, -0.5);
+    const L cx = std::cos((L)kx), cy = std::cos((L)ky);
+    check(std::fabs((double)((L)E - (-0.5L + 2 * (cx + cy) + 4 * (L)-0.3 * cx * cy))) <= 1.5e-15, "line energy", kx, E);
+    check(E == line_energy_grad(kx, ky, 1.0, -0.3, -0.5, gx, gy), "line energy with gradients", kx, E);
+    check(std::fabs((double)((L)gx - (2 + 4 * (L)-0.3 * cy) * std::sin((L)kx))) <= 1e-15, "gradient", kx, gx);
+  }
+  double s, c;
+  cw_sincos(0.0, s, c);
+  check(s == 0.0 && c == 1.0, "sincos(0)", 0.0, s);
+  for (double k : {32.0, -33.5, 100.0, 1e5}) {                             // the out-of-line reduction
+    check(std::fabs(cw_cos(k) - std::cos(k)) <= 3e-16 + 1e-20 * k * k, "cos far", k, cw_cos(k));
+    check(std::fabs(line_energy(k, 1.0, 1.0, 0.0, 0.0) - 2 * (std::cos(k) + std::cos(1.0))) <= 2e-15, "far line", k, 0.0);
+  }
+  for (double k : {inf, -inf, std::nan("")})
+    check(std::isnan(cw_cos(k)) && std::isnan(line_energy(1.0, k, 1.0, 0.0, 0.0)), "not finite", k, cw_cos(k));
+}
+
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
   if (!std::strcmp(what, "rcp")) test_rcp();
   if (!std::strcmp(what, "exp")) test_exp();
+  if (!std::strcmp(what, "trig")) test_trig();
   std::printf("%d failures\n", failures);
   return failures != 0;
 }

@@ -22,7 +22,7 @@ def cases(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["rcp", "exp"])
+@pytest.mark.parametrize("what", ["rcp", "exp", "trig"])
 def test_fixed_point_function(cases, what):
     """Within 0.502 ulp (reciprocal), 0.51 ulp (e^t), 0.75 ulp (e^t - 1), 8e-17 absolute (cos, sin)."""
     r = subprocess.run([str(cases), what], capture_output=True, text=True)
