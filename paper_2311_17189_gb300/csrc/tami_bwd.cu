@@ -85,16 +85,16 @@ __device__ __forceinline__ void bwd_phase2(const TableHeader& H, int n_f, long l
     for (int c = 0; c < H.n_cden; ++c) {
       const double Dr = XR_ZERO ? b[c] : fma(cden_a[c], Xr, b[c]);
       const double r = rcp(fma(Dr, Dr, AXI2[c * n_f + f]));
-      vre[c] = Dr * r;
-      vim[c] = -AXI[c * n_f + f] * r;
+      vre[c] = imul(Dr, r);
+      vim[c] = neg_bits(imul(AXI[c * n_f + f], r));
       U_re[c] = 0.0;
       U_im[c] = 0.0;
     }
     for (int k = 0; k < H.n_pnode; ++k) {
       const int src = pnode[2 * k], c = pnode[2 * k + 1];
       const double ar = vre[src], ai = vim[src], br = vre[c], bi = vim[c];
-      vre[H.n_cden + k] = fma(ar, br, -ai * bi);
-      vim[H.n_cden + k] = fma(ar, bi, ai * br);
+      vre[H.n_cden + k] = fma(ar, br, neg_bits(imul(ai, bi)));
+      vim[H.n_cden + k] = fma(ar, bi, imul(ai, br));
     }
     double vr = 0.0, vi = 0.0;                    // fused pass: the sample's value sum_h W_h R_h
     if (FWD) vr = H.g2_const ? W2[0] : 0.0;
@@ -114,8 +114,8 @@ __device__ __forceinline__ void bwd_phase2(const TableHeader& H, int n_f, long l
     }
     double dvr = 0.0, dvi = 0.0;
     for (int c = 0; c < H.n_cden; ++c) {
-      const double Zr = fma(vre[c], U_re[c], -vim[c] * U_im[c]);
-      const double Zi = fma(vre[c], U_im[c], vim[c] * U_re[c]);
+      const double Zr = fma(vre[c], U_re[c], neg_bits(imul(vim[c], U_im[c])));
+      const double Zi = fma(vre[c], U_im[c], imul(vim[c], U_re[c]));
       dvr = fma(-cden_a[c], Zr, dvr);
       dvi = fma(-cden_a[c], Zi, dvi);
       bb[c] = fma(ngr, Zr, fma(ngi, Zi, bb[c]));
@@ -235,9 +235,15 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
       kx[H.m] = P.kx;
       ky[H.m] = P.ky;
       auto line_momentum = [&](int r, double& ax, double& ay) {
-        ax = 0.0;
-        ay = 0.0;
-        for (int q = lm_ptr[r]; q < lm_ptr[r + 1]; ++q) {
+        int q = lm_ptr[r];
+        const int q1 = lm_ptr[r + 1];
+        ax = ay = 0.0;
+        if (q < q1) {
+          ax = coef_mul(lm_c[q], kx[lm_l[q]]);
+          ay = coef_mul(lm_c[q], ky[lm_l[q]]);
+          ++q;
+        }
+        for (; q < q1; ++q) {
           const double cf = lm_c[q];
           const int l = lm_l[q];
           ax = fma(cf, kx[l], ax);
@@ -257,8 +263,10 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
     }
     double x[kBwCombos];
     for (int u = 0; u < H.n_combo; ++u) {
-      double v = 0.0;
-      for (int q = combo_ptr[u]; q < combo_ptr[u + 1]; ++q) v = fma(combo_c[q], E[combo_j[q]], v);
+      int q = combo_ptr[u];
+      const int q1 = combo_ptr[u + 1];
+      double v = q < q1 ? coef_mul(combo_c[q], E[combo_j[q]]) : 0.0;
+      for (++q; q < q1; ++q) v = fma(combo_c[q], E[combo_j[q]], v);
       x[u] = v;
     }
     double fv[kBwFv], fvd[kBwFv];
@@ -276,13 +284,12 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
         const int dst = op.x & kOpbDstMask, ref = op.y >> kOpbRefShift;
         const bool leaf = op.x & kOpbLeaf;
         const double a = leafA[leaf ? ref : 0], b = val[leaf ? 0 : ref];
-        const double addend = (op.x & kOpbFirst) ? 0.0 : val[dst];
-        val[dst] = fma(fv[op.y & kOpbFvMask], leaf ? a : b, addend);
+        val[dst] = dag_step(fv[op.y & kOpbFvMask], leaf ? a : b, val[dst], op.x & kOpbFirst);
       }
       double ft = val[g1_node[gi]];
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q) {
         const double r = rr[g1rd[2 * q]];
-        for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) ft *= r;
+        for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) ft = imul(ft, r);
       }
       W1[gi] = ft;
       W2[g1_tgt[gi]] += ft;
@@ -296,7 +303,7 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
     double Wb2[kBwG2], bb[kBwCden], pW[kBwG2cd];
     for (int h = 0; h < H.n_g2; ++h) {
       Wb2[h] = 0.0;
-      for (int q = g2[h]; q < g2[h + 1]; ++q) pW[q] = g2cd_p[q] * W2[h];
+      for (int q = g2[h]; q < g2[h + 1]; ++q) pW[q] = coef_mul(g2cd_p[q], W2[h]);
     }
     for (int c = 0; c < H.n_cden; ++c) bb[c] = 0.0;
     if (xr_zero)

@@ -752,6 +752,25 @@ static __device__ __noinline__ double fermi_poly(int k, double g, double h, doub
   return -b4 * beta * gh * (h2 * h2 - 26.0 * g * h2 * h + 66.0 * g2 * h2 - 26.0 * g2 * g * h + g2 * g2);
 }
 
+// -v by its sign bit (no FP64 instruction)
+__device__ __forceinline__ double neg_bits(double v) {
+  return __hiloint2double(__double2hiint(v) ^ (int)0x80000000u, __double2loint(v));
+}
+
+// c v for a table coefficient c (the same in every thread): the tables' +-1 are a copy or a sign flip
+__device__ __forceinline__ double coef_mul(double c, double v) {
+  const int hi = __double2hiint(c);
+  if ((hi & 0x7FFFFFFF) == 0x3FF00000 && __double2loint(c) == 0) return hi < 0 ? neg_bits(v) : v;
+  return __dmul_rn(c, v);
+}
+
+// One pole-DAG step F a + v, or F a for a node's first child (the same flag in every thread): a
+// product, which the integer pipes take
+__device__ __forceinline__ double dag_step(double F, double a, double v, int first) {
+  if (first) return imul(F, a);
+  return fma(F, a, v);
+}
+
 // Fermi values of one segment of the term table: one energy combination x and one sigma, every
 // value g_sigma^(k)(+-x) that the terms use (k = 0 first).  y = e^{-beta|x|} keeps the tails exact;
 // the Bose-type segments (sigma = -1) take 1 - y = -(e^t - 1) from the same exponential.  With
@@ -762,13 +781,13 @@ __device__ __forceinline__ void fermi_segment(const int* seg, const int* fvr, co
                                               double* fv, double* fvd) {
   const double xv = x[seg[0]];
   double em = 0.0;
-  const double y = exp_neg<BOSE>(-beta * fabs(xv), em);
-  const double rD = rcp(BOSE ? -em : 1.0 + y);
-  const double t2 = (BOSE ? -y : y) * rD;
+  const double y = exp_neg<BOSE>(neg_bits(imul(beta, fabs(xv))), em);
+  const double rD = rcp(BOSE ? neg_bits(em) : 1.0 + y);
+  const double t2 = imul(BOSE ? neg_bits(y) : y, rD);
   const bool neg = __double_as_longlong(xv) <= 0;   // xv <= 0 (+0, -0 and negatives), on the ALU
   const double g = neg ? rD : t2, h = neg ? t2 : rD;   // g_sigma(x) and g_sigma(-x)
   double d1 = 0.0;
-  if (DUAL) d1 = -beta * (g * h);
+  if (DUAL) d1 = neg_bits(imul(beta, imul(g, h)));
   for (int v = seg[2]; v < seg[3]; ++v) {
     fv[v] = fvr[2 * v] > 0 ? g : h;
     if (DUAL) fvd[v] = d1;
