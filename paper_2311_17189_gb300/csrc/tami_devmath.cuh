@@ -406,7 +406,10 @@ static __device__ __noinline__ double line_energy_far(double kx, double ky, doub
   return E + bad;
 }
 
-__device__ __forceinline__ double line_energy(double kx, double ky, double t, double tp, double mu) {
+#ifndef TAMI_LINE_INLINE   // the generated kernels call one out-of-line copy
+#define TAMI_LINE_INLINE __forceinline__
+#endif
+__device__ TAMI_LINE_INLINE double line_energy(double kx, double ky, double t, double tp, double mu) {
   double gx, gy;
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<false>(kx, ky, t, tp, mu, gx, gy);
   return line_energy_near<false>(kx, ky, t, tp, mu, gx, gy);
@@ -414,7 +417,7 @@ __device__ __forceinline__ double line_energy(double kx, double ky, double t, do
 
 // Energy of a line that carries k_ext, with the factors G = (2t + 4t' cos K_perp) sin K of
 // dE/dK = -G for both components (one sincos per component); E has line_energy's bits.
-__device__ __forceinline__ double line_energy_grad(double kx, double ky, double t, double tp, double mu, double& gx,
+__device__ TAMI_LINE_INLINE double line_energy_grad(double kx, double ky, double t, double tp, double mu, double& gx,
                                                    double& gy) {
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<true>(kx, ky, t, tp, mu, gx, gy);
   return line_energy_near<true>(kx, ky, t, tp, mu, gx, gy);

@@ -26,7 +26,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
-#include <regex>
 #include <functional>
 #include <atomic>
 #include <memory>
@@ -173,45 +172,24 @@ enum { kKindFused = kJitKindFused, kKindFwd = kJitKindFwd, kKindBwd = kJitKindBw
        kKinds = 4 };
 const char* const kKernelName[kKinds] = {"tami_jit_fused", "tami_jit_fwd", "tami_jit_bwd", "tami_jit_energy"};
 
-// Products of the frequency loop on the integer pipes (imul of tami_devmath.cuh, bit for bit the
-// FP64 unit's product), unless $TAMI_JIT_INTARITH is "0".  On this GPU the FP64 unit bounds the
-// specialised kernels while the integer units are mostly idle, and the two run concurrently; the
-// loop's products, which feed only fmas, move there.  Measured: the order-4 bench step 59.4 ->
-// 54.0 ms.  Not for large tables (over 256 pole-DAG ops), whose kernels already wait on instruction
-// fetch and whose frequency loop runs few times (order 5: 1.054 -> 1.074 s, order 6: 0.80 ->
-// 0.85 s with it); nor in the per-sample code, whose many live values would spill more than the
-// move gains (measured 40 % slower).
-// The adjoint kinds' frequency loop reads its per-sample inputs (the group weights W, the products
-// p W and the frequency-free parts b of the denominators) from shared memory, [value][thread],
-// through volatile loads that the compiler cannot hoist back into registers: the loop body then
-// fits more of its working values in the 64 registers and spills less (order-4 fused step 53.4 ->
-// 49.5 ms, order-3 real-axis workload 108.8 -> 90.9 ms; the plain forward, with fewer live values,
-// gains nothing; the running sums Wbar and b-adjoint there as well measured 0.3 % slower).  $TAMI_JIT_SMEMVALS=0 keeps
-// them in registers.  The slots sit in dynamic shared memory after the reduction buffer; tables
-// with more than 24 such values per thread keep them in registers (24 x 8 B x 1024 threads of a
-// lockstep SM = 192 KB).
-int loop_value_count(const TableHeader& h) { return h.n_g2 + h.n_g2cd + h.n_cden; }
-bool smem_loop_values(const TableHeader& h, bool adj, int block) {
-  const char* e = std::getenv("TAMI_JIT_SMEMVALS");
-  (void)block;
-  return adj && !(e && !std::strcmp(e, "0")) && loop_value_count(h) <= 24;
-}
-
-// Threads per block of a specialised kernel.  The Monte Carlo kinds run in lockstep blocks: 512
-// threads ($TAMI_JIT_LOCKSTEP: 256, 512 or 1024), two blocks per SM, whose warps meet at a barrier
-// every $TAMI_JIT_SYNC_OPS pole-DAG steps (default 32) in the straight-line per-sample code, so
-// that the warps of an SM fetch the same stretch of code at a time instead of spreading over the
-// whole kernel.  A large table's kernel is far larger than the instruction caches: the order-6
-// table's fused step went from 790 to 677 ms (it had waited mostly on instruction fetch); the
-// order-4 step 49.7 -> 48.2 ms, order 3 on the real axis 91.1 -> 86.4 ms, order 5 1.029 ->
-// 1.020 s, against 128-thread blocks without barriers.  The energy-input kind (no reduction, short
-// code) keeps 128-thread blocks.
+// Threads per block of a specialised kernel.  The Monte Carlo kinds run in lockstep blocks, whose
+// warps meet at a barrier after the line energies and every $TAMI_JIT_SYNC_OPS pole-DAG steps
+// (default 32) in the straight-line per-sample code, so that the warps of an SM fetch the same
+// stretch of code at a time instead of spreading over the whole kernel, which is far larger than
+// the instruction caches (order-6 step, 128-thread blocks without barriers -> 512: 790 -> 677 ms).
+// The forward takes one block of 1024 threads per SM (order 4, 2^22 samples x 16 frequencies: 6.68
+// -> 6.35 ms against 512; order 5 2.88 -> 2.84 ms; order 2 2.33 -> 2.29 ms); the adjoint kinds two
+// of 512 (order 3, 2^21 samples x 256 frequencies: 38.6 against 40.2 ms, where a block of 1024
+// leaves half of its last round empty; order 5 6.41 against 6.55 ms).  $TAMI_JIT_LOCKSTEP (256, 512,
+// 1024) sets it for every Monte Carlo kind.  The energy-input kind (no reduction, short code) keeps
+// 128-thread blocks.
 int lockstep_block(const TableHeader& h, int kind) {
   (void)h;
   if (kind == kKindEnergy) return kJitBlock;
   const char* e = std::getenv("TAMI_JIT_LOCKSTEP");
-  const int b = e ? std::atoi(e) : 512;
-  return (b == 256 || b == 1024) ? b : 512;
+  const int b = e ? std::atoi(e) : 0;
+  if (b == 256 || b == 512 || b == 1024) return b;
+  return kind == kKindFwd ? 1024 : 512;
 }
 // Blocks per SM the kernel is compiled for: 1024 threads per SM, 64 registers each.  (128
 // registers at 512 threads per SM halve the large tables' spills and change no step by more than
@@ -243,19 +221,23 @@ bool keep_rr() {
   return !(e && !std::strcmp(e, "0"));
 }
 
-// The per-sample products of tables up to 256 pole-DAG ops (group weights, Fermi segments, the
-// reverse sweep's first adjoint terms, the real denominators' adjoints) run on the integer pipes
-// as well, with the call-free imul_ftz (IEEE products for normal values; subnormals flush to
-// zero): order-4 step 48.07 -> 47.22 ms.  Larger tables keep them on the FP64 unit: there the
-// integer product's registers double the spills (order 6: 663 -> 730 ms).  $TAMI_JIT_PSMUL=0 keeps
-// every table's per-sample products on the FP64 unit, $TAMI_JIT_PSMUL=all moves them for every table,
-// $TAMI_JIT_PSMUL=fwd every table's forward part (values and weights; the reverse sweep keeps the
-// default).
-bool ps_products(const TableHeader& h, bool reverse = false) {
+// The share of the per-sample products (group weights, Fermi segments, the reverse sweep's first
+// adjoint terms, the real denominators' adjoints) that goes to the integer pipes, as the call-free
+// imul_ftz (IEEE products for normal values; subnormals flush to zero).  The forward part's
+// exponentials, reciprocals and cosines occupy these pipes already, so tables up to 256 pole-DAG
+// ops move the balanced share (order 4, fused, 2^22 samples x 16 frequencies: 16.23 ms, none 16.97,
+// all 17.4), larger ones, whose registers spill, none (order 5 fused 6.42 against 6.66 ms with 30 %).
+// The reverse sweep keeps its products on the FP64 unit (order 4 17.9 ms with all of them moved,
+// order 5 6.99 against 6.42 ms): there the integer product's registers cost more than its slots.
+// $TAMI_JIT_PSMUL=0 keeps every product on the FP64 unit, =all moves every one, =fwd every one of
+// the forward part.
+struct PsShare { double fwd = 1.0, rev = 1.0; };
+PsShare ps_share(PsShare balanced) {
   const char* e = std::getenv("TAMI_JIT_PSMUL");
-  if (e && !std::strcmp(e, "all")) return true;   // every table ($TAMI_JIT_PSMUL=all)
-  if (e && !std::strcmp(e, "fwd") && !reverse) return true;   // every table's forward part
-  return h.n_ops <= 256 && !(e && !std::strcmp(e, "0"));
+  if (e && !std::strcmp(e, "all")) return PsShare{1.0, 1.0};
+  if (e && !std::strcmp(e, "0")) return PsShare{0.0, 0.0};
+  if (e && !std::strcmp(e, "fwd")) balanced.fwd = 1.0;
+  return balanced;
 }
 // The reverse sweep's sums (combination, Fermi-value and energy adjoints, each segment's sum) take
 // their first term as an assignment, a copy or a product, instead of an add or fma onto 0.0 that the
@@ -270,10 +252,16 @@ bool ps_first_steps() {
   const char* e = std::getenv("TAMI_JIT_PSFIRST");
   return !(e && !std::strcmp(e, "0"));
 }
-// a * b, on the integer pipes where the per-sample products go there
-std::string pmul(bool ps, const std::string& a, const std::string& b) {
-  return ps ? "imul_ftz(" + a + ", " + b + ")" : a + " * " + b;
-}
+// Spreads a share evenly over a sequence of products: next() says whether the next one is in it.
+struct Spread {
+  double share = 1.0, due = 0.0;
+  bool next() {
+    due += share;
+    if (due < 1.0 - 1e-9) return false;
+    due -= 1.0;
+    return true;
+  }
+};
 
 // The frequency loop's products (1/D = D r, the trie's complex products, Z, the sums' first terms)
 // run on the integer pipes with imul, for every table: with 32 frequencies the 85 order-2..5
@@ -293,18 +281,23 @@ int count_of(const std::string& s, const char* what) {
   return n;
 }
 
-// The share of a loop's products that goes to the integer pipes, so that these and the FP64 unit
-// finish together: with `loop` the generated loop whose products are all imul, and times in FP64
-// instructions (67 clocks of an SM quarter each), a product costs the integer pipes 1.1, a
-// reciprocal 0.95 and the loop's own indexing, loads and stores about 1 (measured one by one:
-// imul 74 clocks, rcp 63).  Loops with many sums keep every product on the integer pipes; the
-// evaluation example's (one denominator, no sums) moves three of its four back: 1.155 -> 0.872 ms
-// for 10^6 rows and 100 frequencies, two external frequencies (400 000 rows) 5.13 -> 4.79 ms.
-double loop_share(const std::string& loop) {
-  const double fp = count_of(loop, "fma(") + count_of(loop, " += ");
-  const double ints = 0.95 * count_of(loop, "rcp(") + 1.0;
-  const double products = count_of(loop, "imul("), cost = 1.1;
+// The share of the products of a piece of generated code that goes to the integer pipes, so that
+// these and the FP64 unit finish together, from the code written with all of them there: times in
+// FP64 instructions (67 clocks of an SM quarter), measured one by one -- imul 74 clocks, imul_ftz
+// 84, rcp 63, a Fermi segment's exponential and reciprocal 253 (Bose-type 313) beside its add, a
+// line energy 373 beside its two fmas, with gradients 655 beside six, a Philox draw about 240
+// beside its two conversions and fmas; `other` the indexing, loads and stores.
+double balanced_share(const std::string& code, double other) {
+  const double seg_f = count_of(code, "= tami_seg_fermi("), seg_b = count_of(code, "= tami_seg_bose(");
+  const double line = count_of(code, "= line_energy("), grad = count_of(code, "= line_energy_grad(");
+  const double draws = count_of(code, "philox4x32_10(");
+  const double fp = count_of(code, "fma(") + count_of(code, " += ") + count_of(code, " -= ") + seg_f + 2 * line +
+                    6 * grad + 4 * draws;
+  const double ints = 0.95 * count_of(code, "rcp(") + 3.8 * seg_f + 4.7 * seg_b + 5.6 * line + 9.8 * grad +
+                      3.6 * draws + other;
+  const double loop = count_of(code, "imul("), ps = count_of(code, "imul_ftz("), products = loop + ps;
   if (products <= 0.0) return 1.0;
+  const double cost = (1.1 * loop + 1.25 * ps) / products;
   const double on_fp = (ints + cost * products - fp) / (1.0 + cost);
   return std::min(1.0, std::max(0.0, 1.0 - on_fp / products));
 }
@@ -313,15 +306,9 @@ double loop_share(const std::string& loop) {
 void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
   const TableHeader& h = t.h;
   const bool ia = int_products(h);
-  const bool ps = ps_products(h) && kind != kKindEnergy;
-  auto PM = [&](const std::string& a, const std::string& b) { return pmul(ps, a, b); };
-  double due = 0.0;
+  Spread spread{share};
   auto MUL = [&](const std::string& a, const std::string& b) {
-    if (!ia) return PM(a, b);
-    due += share;
-    if (due < 1.0 - 1e-9) return a + " * " + b;
-    due -= 1.0;
-    return "imul(" + a + ", " + b + ")";
+    return ia && spread.next() ? "imul(" + a + ", " + b + ")" : a + " * " + b;
   };
   auto NEG = [&](const std::string& a) {   // sign flip (no arithmetic)
     return "__longlong_as_double(__double_as_longlong(" + a + ") ^ (long long)0x8000000000000000ull)";
@@ -422,16 +409,25 @@ bool jit_supported(const TableHeader& h, int kind, std::string* why) {
   return true;
 }
 
-// CUDA C++ source of the specialised kernel of one kind for one table.
-std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind) {
-  // Large tables (over 256 pole-DAG ops) are written out into more code than the instruction
-  // caches hold; their Fermi segments call one out-of-line copy of the exponential, reciprocal and
-  // selects (smaller code; the largest order-5 table: 2.6 % faster, the order-4 table unchanged).
-  const bool seg_calls = h.n_ops > 256;
+namespace {
+
+// CUDA C++ source of the specialised kernel of one kind for one table, with the given shares of the
+// per-sample products on the integer pipes; part: where its forward part and its reverse sweep
+// begin and end.
+std::string write_source(const TableHeader& h, const unsigned char* blob, int kind, PsShare share, size_t (*part)[2]) {
+  // The kernels are written out into more code than the instruction caches hold, so their Fermi
+  // segments call one out-of-line copy of the exponential, reciprocal and selects, and their lines
+  // one of the line energy (the barrier after the lines, below, has the block's warps start the
+  // rest together).  Inline, without the barrier, the warps waited on instruction fetch: five
+  // bubbles fused 15.6 -> 11.7 ms per 2^22 samples, order-4 forward 9.03 -> 7.17 ms, order-4
+  // fused 18.2 -> 17.9 ms, the order-4 energy input 2.80 -> 2.67 ms.
   // (the energy-input kind keeps its per-row products on the FP64 unit: 1.093 -> 1.125 ms with them
   // on the integer pipes on the paper's energy-input example)
-  bool ps = ps_products(h) && kind != kKindEnergy;   // the reverse sweep may set it otherwise
-  auto PM = [&](const std::string& a, const std::string& b) { return pmul(ps, a, b); };
+  if (kind == kKindEnergy) share = PsShare{0.0, 0.0};
+  Spread spread{share.fwd};
+  auto PM = [&](const std::string& a, const std::string& b) {
+    return spread.next() ? "imul_ftz(" + a + ", " + b + ")" : a + " * " + b;
+  };
   const Table t{h, blob};
   const bool energy = kind == kKindEnergy;
   const bool fwd = kind != kKindBwd, adj = kind == kKindFused || kind == kKindBwd;
@@ -470,6 +466,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
   };
   o("// generated by libtami for one flattened term table, one sample per thread: %s",
     kind == kKindFused ? "forward + adjoint" : kind == kKindFwd ? "forward" : kind == kKindBwd ? "adjoint" : "energy input");
+  o("#define TAMI_LINE_INLINE static __noinline__");
   o("#include \"tami_devmath.cuh\"");
   o("using namespace tami::dev;");
   if (h.n_cden > 0) {
@@ -486,8 +483,8 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     for (int i = 0; i < h.n_xk * h.n_ext; ++i) v += (i ? ", " : "") + lit(xvec[i]);
     o("__device__ const double kJitXvec[%d] = {%s};", h.n_xk * h.n_ext, v.c_str());
   }
-  if (seg_calls) {
-    // one out-of-line copy of a Fermi segment's exponential, reciprocal and selects (smaller code)
+  {
+    // one out-of-line copy of a Fermi segment's exponential, reciprocal and selects
     for (int bose = 0; bose < 2; ++bose) {
       o("static __device__ __noinline__ double2 tami_seg_%s(double xv, double beta) {", bose ? "bose" : "fermi");
       o("  double em = 0.0;");
@@ -526,7 +523,6 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
   } else {
     o("  double* Xs = smem; double* Gs = Xs + 2 * n_f; double* AXI = Gs + 2 * n_f; double* AXI2 = AXI + %d * n_f;", h.n_cden);
     o("  double* red = AXI2 + %d * n_f;", h.n_cden);
-    if (smem_loop_values(h, adj, B)) o("  volatile double* jsv = red + %d;", B);   // after the [warp][32] buffer
     o("  (void)AXI; (void)AXI2; (void)G; (void)ps_dX; (void)ps_grad; (void)ps_v; (void)saved;");
     o("  for (int i = tid; i < 2 * n_f; i += %d) { Xs[i] = X[i]; Gs[i] = %s; }", B, adj ? "G[i]" : "0.0");
   }
@@ -557,6 +553,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
   o("  }");
   o("  const long long n_tiles = (n + %d) / %d;", B - 1, B);
   o("  for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {");
+  part[0][0] = o.s.size();
   if (ls) {
     // every thread reaches every barrier: a lane past the end runs the last sample again and
     // neither adds nor writes
@@ -624,6 +621,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
   }
   }  // !energy
   o("    }");
+  if (ls) o("    __syncthreads();");
   // ---- energy combinations
   for (int u = 0; u < h.n_combo; ++u) {
     int q0 = combo_ptr[u];
@@ -645,21 +643,11 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     bool has_k1 = false;
     for (int v = sgm[3]; v < sgm[4]; ++v) has_k1 |= fvr[2 * v + 1] == 1;
     const std::string d1 = (adj || has_k1)
-        ? PM("-beta", ps ? PM("sg" + std::to_string(b) + "_g", "sg" + std::to_string(b) + "_h")
-                         : "(sg" + std::to_string(b) + "_g * sg" + std::to_string(b) + "_h)")
+        ? PM("-beta", "(" + PM("sg" + std::to_string(b) + "_g", "sg" + std::to_string(b) + "_h") + ")")
         : std::string("0.0");
     o("    double sg%d_g, sg%d_h, sg%d_d1;", b, b, b);
-    if (seg_calls) {
-      o("    { const double2 gh = tami_seg_%s(x%d, beta);", bose ? "bose" : "fermi", sgm[0]);
-      o("      sg%d_g = gh.x; sg%d_h = gh.y; sg%d_d1 = %s; }", b, b, b, d1.c_str());
-    } else {
-    o("    { const double xv = x%d; double em = 0.0;", sgm[0]);
-    o("      const double y = exp_neg<%s>(%s, em); (void)em;", bose ? "true" : "false", PM("-beta", "fabs(xv)").c_str());
-    o("      const double rD = rcp(%s);", bose ? "-em" : "1.0 + y");
-    o("      const double t2 = %s;", PM(bose ? "(-y)" : "(y)", "rD").c_str());
-    o("      const bool neg = __double_as_longlong(xv) <= 0;");
-    o("      sg%d_g = neg ? rD : t2; sg%d_h = neg ? t2 : rD; sg%d_d1 = %s; }", b, b, b, d1.c_str());
-    }
+    o("    { const double2 gh = tami_seg_%s(x%d, beta);", bose ? "bose" : "fermi", sgm[0]);
+    o("      sg%d_g = gh.x; sg%d_h = gh.y; sg%d_d1 = %s; }", b, b, b, d1.c_str());
     for (int v = sgm[2]; v < sgm[3]; ++v) {
       o("    const double fv%d = sg%d_%c;", v, b, fvr[2 * v] > 0 ? 'g' : 'h');
       if (adj) o("    const double fvd%d = sg%d_d1;", v, b);
@@ -668,7 +656,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     // with k = 1 values (an h value's is -d2)
     if (adj && has_k1)
       o("    const double sg%d_d2 = %s;", b,
-        PM(PM("-beta", "sg" + std::to_string(b) + "_d1"), "(sg" + std::to_string(b) + "_h - sg" + std::to_string(b) + "_g)").c_str());
+        PM("(" + PM("-beta", "sg" + std::to_string(b) + "_d1") + ")", "(sg" + std::to_string(b) + "_h - sg" + std::to_string(b) + "_g)").c_str());
     for (int v = sgm[3]; v < sgm[4]; ++v) {
       const bool pos = fvr[2 * v] > 0;
       const int k = fvr[2 * v + 1];
@@ -705,8 +693,8 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
       const std::string add = q.parent < 0 ? "0.0" : "pv" + std::to_string(q.parent);
       if (q.parent < 0 && !q.node && (c == 1.0 || c == -1.0))
         o("    const double pv%d = %sfv%d;", k, c > 0 ? "" : "-", q.fv);   // +-F, no arithmetic
-      else if (q.parent < 0 && ps && ps_first_steps())   // a chain's first step is a product
-        o("    const double pv%d = %s;", k, PM("fv" + std::to_string(q.fv), opnd).c_str());
+      else if (q.parent < 0 && ps_first_steps() && spread.next())   // a chain's first step is a product
+        o("    const double pv%d = imul_ftz(fv%d, %s);", k, q.fv, opnd.c_str());
       else
         o("    const double pv%d = fma(fv%d, %s, %s);", k, q.fv, opnd.c_str(), add.c_str());
       step_sync();
@@ -717,7 +705,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q)
         for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) {
           if (first) o("    double RR_%d = rr%d;", gi, g1rd[2 * q]);
-          else if (ps) o("    RR_%d = imul_ftz(RR_%d, rr%d);", gi, gi, g1rd[2 * q]);
+          else if (spread.next()) o("    RR_%d = imul_ftz(RR_%d, rr%d);", gi, gi, g1rd[2 * q]);
           else o("    RR_%d *= rr%d;", gi, g1rd[2 * q]);
           first = false;
         }
@@ -726,7 +714,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
       o("    double W1_%d = %s;", gi, root_pv(gi).c_str());
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q)
         for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) {
-          if (ps) o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
+          if (spread.next()) o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
           else o("    W1_%d *= rr%d;", gi, g1rd[2 * q]);
         }
     }
@@ -740,7 +728,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     for (int g = 0; g < h.n_g2; ++g) {
       o("    double Wb2_%d = 0.0;", g);
       for (int q = g2[g]; q < g2[g + 1]; ++q) {
-        if (ps && (g2cd_p[q] == 1.0 || g2cd_p[q] == -1.0))
+        if (g2cd_p[q] == 1.0 || g2cd_p[q] == -1.0)
           o("    const double pW%d = %sW2_%d;", q, g2cd_p[q] > 0 ? "" : "-", g);
         else
           o("    const double pW%d = %s;", q, PM(lit(g2cd_p[q]), "W2_" + std::to_string(g)).c_str());
@@ -748,51 +736,23 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     }
     for (int c = 0; c < h.n_cden; ++c) o("    double bb%d = 0.0;", c);
   }
-  // ---- phase 2 over frequencies (the adjoint kinds' loop inputs in shared memory, see
-  // smem_loop_values)
-  const bool sv = smem_loop_values(h, adj, B);
-  const int n_sv = h.n_g2 + h.n_g2cd + h.n_cden;
-  if (sv) {
-    for (int g = 0; g < h.n_g2; ++g) o("    jsv[%d * %d + tid] = W2_%d;", g, B, g);
-    for (int q = 0; q < h.n_g2cd; ++q) o("    jsv[%d * %d + tid] = pW%d;", h.n_g2 + q, B, q);
-    for (int c = 0; c < h.n_cden; ++c) o("    jsv[%d * %d + tid] = b%d;", n_sv - h.n_cden + c, B, c);
-  }
-  const size_t loop0 = o.s.size();
+  // ---- phase 2 over frequencies
+  part[0][1] = o.s.size();
   auto loop = [&](bool xr_zero) {
     Out whole;
     emit_phase2(whole, t, kind, xr_zero, 1.0);
-    emit_phase2(o, t, kind, xr_zero, loop_share(whole.s));
+    emit_phase2(o, t, kind, xr_zero, balanced_share(whole.s, 1.0));
   };
   o("    if (xr_zero) {");
   loop(true);
   o("    } else {");
   loop(false);
   o("    }");
-  if (sv) {
-    std::string loop = o.s.substr(loop0);
-    auto rename = [&](const char* pat, int base) {
-      const std::regex re(pat);
-      std::string out;
-      std::sregex_iterator it(loop.begin(), loop.end(), re), end;
-      size_t last = 0;
-      for (; it != end; ++it) {
-        out += loop.substr(last, it->position() - last);
-        out += "jsv[" + std::to_string(base + std::stoi((*it)[1].str())) + " * " + std::to_string(B) + " + tid]";
-        last = it->position() + it->length();
-      }
-      out += loop.substr(last);
-      loop.swap(out);
-    };
-    rename("\\bW2_(\\d+)\\b", 0);
-    rename("\\bpW(\\d+)\\b", h.n_g2);
-    rename("\\bb(\\d+)\\b", n_sv - h.n_cden);
-    o.s.resize(loop0);
-    o.s += loop;
-  }
   if (adj) {
     if (h.g2_const) o("    Wb2_0 = s_gsum;");
     // ---- reverse sweep
-    ps = ps_products(h, true) && kind != kKindEnergy;
+    part[1][0] = o.s.size();
+    spread = Spread{share.rev};
     const bool ft = first_terms();
     for (int u = 0; u < h.n_combo; ++u) o(ft ? "    double xbar%d;" : "    double xbar%d = 0.0;", u);
     for (int v = 0; v < h.n_fv; ++v) o(ft ? "    double fvbar%d;" : "    double fvbar%d = 0.0;", v);
@@ -819,15 +779,11 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
         const int i = g1rd[2 * q], pw = g1rd[2 * q + 1];
         if (!kept) for (int k = 0; k < pw; ++k) o("      RR *= rr%d;", i);
         const int u = rden[2 * i];
-        if (ps) {   // wb W1 once per group, then one fma per factor
-          if (q == g1[4 * gi + 2]) o("      const double tw = %s;", PM("wb", "W1_" + std::to_string(gi)).c_str());
-          const std::string tp = pw == 1 ? "tw" : PM("tw", lit((double)pw));
-          if (hx[u]) o("      xbar%d = fma(-%s, rr%d, xbar%d);", u, tp.c_str(), i, u);
-          else o("      xbar%d = %s;", u, PM("-" + tp, "rr" + std::to_string(i)).c_str());
-        } else {
-          if (hx[u]) o("      xbar%d -= wb * W1_%d * %s * rr%d;", u, gi, lit((double)pw).c_str(), i);
-          else o("      xbar%d = -(wb * W1_%d * %s * rr%d);", u, gi, lit((double)pw).c_str(), i);
-        }
+        // wb W1 once per group, then one fma per factor
+        if (q == g1[4 * gi + 2]) o("      const double tw = %s;", PM("wb", "W1_" + std::to_string(gi)).c_str());
+        const std::string tp = pw == 1 ? "tw" : PM("tw", lit((double)pw));
+        if (hx[u]) o("      xbar%d = fma(-(%s), rr%d, xbar%d);", u, tp.c_str(), i, u);
+        else o("      xbar%d = %s;", u, PM("-(" + tp + ")", "rr" + std::to_string(i)).c_str());
         hx[u] = 1;
       }
       if (has[rp]) o("      bp%d = fma(%swb, RR, bp%d);", rp, rs, rp);
@@ -907,6 +863,7 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
     o("      gmu += mub; gkx += kxb; gky += kyb;");
     o("      if (ps_grad) { ps_grad[3 * s] = mub; ps_grad[3 * s + 1] = kxb; ps_grad[3 * s + 2] = kyb; }");
     o("    }");
+    part[1][1] = o.s.size();
   }
   o("  }");
   if (energy) {   // every value is an output; nothing is reduced
@@ -940,6 +897,15 @@ std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind
   o("  }");
   o("}");
   return o.s;
+}
+
+}  // namespace
+
+std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind) {
+  size_t part[2][2] = {{0, 0}, {0, 0}};
+  const std::string whole = write_source(h, blob, kind, PsShare{1.0, 1.0}, part);
+  auto share = [&](int i) { return balanced_share(whole.substr(part[i][0], part[i][1] - part[i][0]), 0.0); };
+  return write_source(h, blob, kind, ps_share(PsShare{h.n_ops <= 256 ? share(0) : 0.0, 0.0}), part);
 }
 
 // --------------------------------------------------------------------------- disk cache entries
@@ -1125,9 +1091,7 @@ int jit_prepare(tami_diagram* d, int kind) {
 size_t jit_smem(const TableHeader& h, int kind, int n_f, int block) {
   if (kind == kKindEnergy) return sizeof(double) * (size_t)(2 * h.n_xk + 2 * h.n_cden) * n_f;
   const size_t red = (size_t)block;   // the block reduction's [warp][32] buffer
-  const bool adj = kind == kKindFused || kind == kKindBwd;
-  const size_t jsv = smem_loop_values(h, adj, block) ? (size_t)block * loop_value_count(h) : 0;
-  return sizeof(double) * ((size_t)(4 + 2 * h.n_cden) * n_f + red + jsv);
+  return sizeof(double) * ((size_t)(4 + 2 * h.n_cden) * n_f + red);
 }
 
 int jit_select(tami_diagram* d, int kind, int64_t n, int n_f, bool generic_ok) {
