@@ -709,13 +709,13 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
           else o("    RR_%d *= rr%d;", gi, g1rd[2 * q]);
           first = false;
         }
-      o("    double W1_%d = %s;", gi, PM(root_pv(gi), "RR_" + std::to_string(gi)).c_str());
+      // (imul_ftz: a plain product could be contracted into W2's sum, in one kind and not in another)
+      o("    double W1_%d = imul_ftz(%s, RR_%d);", gi, root_pv(gi).c_str(), gi);
     } else {
       o("    double W1_%d = %s;", gi, root_pv(gi).c_str());
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q)
         for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) {
-          if (spread.next()) o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
-          else o("    W1_%d *= rr%d;", gi, g1rd[2 * q]);
+          o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
         }
     }
     o(has_w2[g1_tgt[gi]] ? "    W2_%d += W1_%d;" : "    W2_%d = W1_%d;", g1_tgt[gi], gi);
