@@ -250,7 +250,7 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
                           tami_stream_t stream);
 
 /* tami_forward without a workspace argument: the same Monte Carlo evaluation and outputs, with
- * its scratch (a status word and the per-block partial sums) taken from a fixed 4 MiB array
+ * its scratch (the per-block partial sums) taken from a fixed 4 MiB array
  * inside libtami instead of memory the caller allocates.  The paper has no counterpart; this
  * entry exists for callers that cannot allocate device memory, e.g. code whose device memory
  * is all owned by a pool fixed at start-up, or loops that must not let cudaMalloc/cudaFree
@@ -264,9 +264,8 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
  *     message; use tami_forward with a workspace for them.
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress, with
  *     that device current); make that first call before any stream capture.
- *   - Every call shares the one array and it keeps the last call's contents; the call clears the
- *     status word itself.  Calls whose work overlaps on the GPU (other streams, other host
- *     threads) race on the array: serialise them.
+ *   - Every call shares the one array and it keeps the last call's contents.  Calls whose work
+ *     overlaps on the GPU (other streams, other host threads) race on the array: serialise them.
  *   - The looked-up address is kept for the life of the process: a device reset
  *     (cudaDeviceReset) while libtami is loaded is not supported with this call.
  *   - It always runs the generic kernel (never a specialised one, whose grid it does not size

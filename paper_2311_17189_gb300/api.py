@@ -34,6 +34,10 @@ def _as_c_pairs(X, device, n_ext=1):
     """complex [n_f] (or [n_f, n_ext]: one row of external frequencies per f) -> contiguous
     float64 [n_f, 2] ([n_f, n_ext, 2]) on `device`."""
     torch = _torch()
+    if (isinstance(X, torch.Tensor) and X.dtype == torch.complex128 and X.is_cuda and X.is_contiguous() and
+            X.dim() == (1 if n_ext == 1 else 2) and not X.is_conj() and X.device == device and
+            (n_ext == 1 or X.shape[1] == n_ext)):
+        return torch.view_as_real(X)       # already in place
     X = torch.as_tensor(X)
     if not torch.is_complex(X):
         X = X.to(torch.complex128)
@@ -88,6 +92,7 @@ class Diagram:
         self._h = h
         self.device = None
         self._ws = None
+        self._n_saved = None
 
     def __del__(self):
         h = getattr(self, "_h", None)
@@ -106,7 +111,7 @@ class Diagram:
     def _dev(self):
         if self.device is None:
             raise L.TamiError(L.TAMI_EINVAL, "diagram not uploaded (call upload)")
-        return f"cuda:{self.device}"
+        return self._device
 
     def jit_prepare(self):
         """Build the specialised kernels of this uploaded diagram now (tami_jit_prepare)."""
@@ -142,6 +147,7 @@ class Diagram:
         with torch.cuda.device(dev):
             L.check(L.lib().tami_upload(self._h, dev, _stream_ptr()))
         self.device = dev
+        self._device = torch.device("cuda", dev)
         return self
 
     # ---------------------------------------------------------------- evaluation
@@ -179,7 +185,12 @@ class Diagram:
     def saved_buffer(self, n):
         """A buffer for forward(save=...) / backward(saved=...): float64 [saved_rows, n]."""
         torch = _torch()
-        return torch.empty((self.info()["saved_rows"], int(n)), dtype=torch.float64, device=self._dev())
+        return torch.empty((self._saved_rows(), int(n)), dtype=torch.float64, device=self._dev())
+
+    def _saved_rows(self):
+        if self._n_saved is None:
+            self._n_saved = self.info()["saved_rows"]
+        return self._n_saved
 
     def forward(self, lattice, seed, offset, n, X, beta, per_sample=False, out=None, save=None):
         """Monte Carlo mean over n momentum samples (Sec. 5.2).  Returns (mean complex [n_f],
@@ -197,7 +208,7 @@ class Diagram:
             mean, var = out
         ps = torch.empty((n_f, n, 2), dtype=torch.float64, device=dev) if per_sample else None
         if save is not None and (save.dtype != torch.float64 or not save.is_contiguous() or
-                                 tuple(save.shape) != (self.info()["saved_rows"], int(n))):
+                                 tuple(save.shape) != (self._saved_rows(), int(n))):
             raise L.TamiError(L.TAMI_EINVAL, "save must be a contiguous float64 [saved_rows, n] tensor")
         ws = self.workspace(n, n_f)
         lat = L.Lattice(*[float(v) for v in lattice])
@@ -227,7 +238,7 @@ class Diagram:
         ps_dX = torch.empty((n_f, n, 2), dtype=torch.float64, device=dev) if per_sample else None
         ps_g = torch.empty((n, 3), dtype=torch.float64, device=dev) if per_sample else None
         if saved is not None and (saved.dtype != torch.float64 or not saved.is_contiguous() or
-                                  tuple(saved.shape) != (self.info()["saved_rows"], int(n))):
+                                  tuple(saved.shape) != (self._saved_rows(), int(n))):
             raise L.TamiError(L.TAMI_EINVAL, "saved must be a contiguous float64 [saved_rows, n] tensor")
         nbytes = ctypes.c_size_t()
         L.check(L.lib().tami_backward_workspace(self._h, int(n), n_f, ctypes.byref(nbytes)))

@@ -46,7 +46,6 @@ struct BwdParams {
   const double* saved;   // [n_rep + 2 n_rep_ext][n] from tami_forward, or null (recompute)
   double* ps_v;          // fused pass: [n_f][n][2] each sample's value, or null
   double* partial;       // [grid][2 n_f + 3]
-  int* status;
   long long wait_limit;   // bound of the first stage of the staging wait
 };
 
@@ -149,9 +148,14 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   extern __shared__ __align__(16) unsigned char smem[];
   const TableHeader& H = P.h;
   const int tid = threadIdx.x;
-  if (!stage_table(smem, P.table, H.off_ops, P.status, P.wait_limit, P.table + H.off_opsb, H.bytes - H.off_opsb))
-    return;
   const int n_f = P.n_f;
+  let_next_kernel_start();
+  __shared__ int s_late;                     // set when the staging wait of this block ran out
+  if (tid == 0) s_late = 0;
+  if (!stage_table(smem, P.table, H.off_ops, &s_late, P.wait_limit, P.table + H.off_opsb, H.bytes - H.off_opsb)) {
+    nan_row(P.partial + (size_t)blockIdx.x * bwd_nval(n_f, FWD), bwd_nval(n_f, FWD));
+    return;
+  }
   double* Xs = reinterpret_cast<double*>(smem + bwd_table_smem(H));
   double* Gs = Xs + 2 * n_f;
   double* AXI = Gs + 2 * n_f;
@@ -400,14 +404,15 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   }
   __syncthreads();
   for (int i = tid; i < nval; i += kBlock) {
-    double v = 0.0;
+    double v = s_late ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;   // late staging: NaN sums
     for (int w = 0; w < kBlock / 32; ++w) v += red[w * nval + i];
     P.partial[(size_t)blockIdx.x * nval + i] = v;
   }
 }
 
 __global__ void __launch_bounds__(kFinBlock) bwd_finalize_kernel(const double* partial, int n_blocks, int n_f, long long n, const double* G,
-                                    const int* status, double* dX, double* grad_omega, double* grad_params) {
+                                    double* dX, double* grad_omega, double* grad_params) {
+  wait_for_previous_kernel();
   // block i < n_f: dSigma/dX_i (two columns); block n_f: the three parameter gradients
   __shared__ double sh[3][kFinBlock];
   const int i = blockIdx.x;
@@ -422,15 +427,12 @@ __global__ void __launch_bounds__(kFinBlock) bwd_finalize_kernel(const double* p
   }
   fixed_tree_sum<3>(s, sh);
   if (threadIdx.x != 0) return;
-  const bool bad = status && *status != 0;
-  const double nan = __longlong_as_double(0x7ff8000000000000ll);
   if (i < n_f) {
-    double re = s[0] / (double)n, im = s[1] / (double)n;
-    if (bad) re = im = nan;
+    const double re = s[0] / (double)n, im = s[1] / (double)n;
     if (dX) { dX[2 * i] = re; dX[2 * i + 1] = im; }
-    if (grad_omega) grad_omega[i] = bad ? nan : fma(G[2 * i], re, G[2 * i + 1] * im);
+    if (grad_omega) grad_omega[i] = fma(G[2 * i], re, G[2 * i + 1] * im);
   } else if (grad_params) {
-    for (int k = 0; k < 3; ++k) grad_params[k] = bad ? nan : s[k] / (double)n;
+    for (int k = 0; k < 3; ++k) grad_params[k] = s[k] / (double)n;
   }
 }
 
@@ -469,25 +471,11 @@ int bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool
     const long long tiles = (n + kBlock - 1) / kBlock;
     return (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
   }
-  int per_sm = 0;
-  if (fwd) {
-    cudaFuncSetAttribute(bwd_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_kernel<false, true>, kBlock, smem) != cudaSuccess)
-      per_sm = 1;
-  } else {
-    // one grid for both adjoint instances (saved rows or recomputation), so that their reductions
-    // group the samples alike and the results agree bit for bit
-    cudaFuncSetAttribute(bwd_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(bwd_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int per_sm_saved = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bwd_kernel<false, false>, kBlock, smem) != cudaSuccess)
-      per_sm = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_saved, bwd_kernel<true, false>, kBlock, smem) !=
-        cudaSuccess)
-      per_sm_saved = 1;
-    if (per_sm_saved < per_sm) per_sm = per_sm_saved;
-  }
-  if (per_sm < 1) per_sm = 1;
+  auto resident = [&](const void* kernel) { return resident_blocks(d->device, kernel, kBlock, smem); };
+  // one grid for both adjoint instances (saved rows or recomputation), so that their reductions
+  // group the samples alike and the results agree bit for bit
+  const int per_sm = fwd ? resident((const void*)bwd_kernel<false, true>)
+                         : std::min(resident((const void*)bwd_kernel<false, false>), resident((const void*)bwd_kernel<true, false>));
   long long tiles = (n + kBlock - 1) / kBlock;
   long long grid = (long long)dp.sms * per_sm;
   if (grid > tiles) grid = tiles;
@@ -498,9 +486,10 @@ int bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool
 // The fused pass's final reduction: block f < n_f sums dv/dX_f and the forward's four sums of f,
 // block n_f the three parameter gradients; fixed tree order.
 __global__ void __launch_bounds__(kFinBlock) fused_finalize_kernel(const double* partial, int n_blocks, int n_f,
-                                                                  long long n, const double* G, const int* status,
-                                                                  double* mean, double* var, double* dX,
+                                                                  long long n, const double* G, double* mean,
+                                                                  double* var, double* dX,
                                                                   double* grad_omega, double* grad_params) {
+  wait_for_previous_kernel();
   __shared__ double sh[6][kFinBlock];
   const int i = blockIdx.x;
   const int nval = bwd_nval(n_f, true);
@@ -517,20 +506,19 @@ __global__ void __launch_bounds__(kFinBlock) fused_finalize_kernel(const double*
   }
   fixed_tree_sum<6>(s, sh);
   if (threadIdx.x != 0) return;
-  const bool bad = status && *status != 0;
-  const double nan = __longlong_as_double(0x7ff8000000000000ll), nn = (double)n;
+  const double nn = (double)n;
   if (i < n_f) {
-    const double re = bad ? nan : s[0] / nn, im = bad ? nan : s[1] / nn;
+    const double re = s[0] / nn, im = s[1] / nn;
     if (dX) { dX[2 * i] = re; dX[2 * i + 1] = im; }
-    if (grad_omega) grad_omega[i] = bad ? nan : fma(G[2 * i], re, G[2 * i + 1] * im);
+    if (grad_omega) grad_omega[i] = fma(G[2 * i], re, G[2 * i + 1] * im);
     const double mr = s[2] / nn, mi = s[3] / nn;
     const double vr = n > 1 ? (s[4] - s[2] * mr) / (nn - 1.0) : 0.0;
     const double vi = n > 1 ? (s[5] - s[3] * mi) / (nn - 1.0) : 0.0;
-    mean[2 * i] = bad ? nan : mr;
-    mean[2 * i + 1] = bad ? nan : mi;
-    if (var) { var[2 * i] = bad ? nan : vr; var[2 * i + 1] = bad ? nan : vi; }
+    mean[2 * i] = mr;
+    mean[2 * i + 1] = mi;
+    if (var) { var[2 * i] = vr; var[2 * i + 1] = vi; }
   } else if (grad_params) {
-    for (int k = 0; k < 3; ++k) grad_params[k] = bad ? nan : s[k] / nn;
+    for (int k = 0; k < 3; ++k) grad_params[k] = s[k] / nn;
   }
 }
 
@@ -547,7 +535,7 @@ int bwd_check(const tami_diagram* d, int n_f) {
   return TAMI_OK;
 }
 
-constexpr size_t kBwStatusBytes = 256;
+constexpr size_t kBwHeadBytes = 256;   // the partial sums start here in a workspace
 
 }  // namespace
 }  // namespace tami
@@ -561,7 +549,7 @@ int tami_backward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, s
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
   const int grid = bwd_grid(d, n_f, n_samples, nullptr, false);
-  *bytes = kBwStatusBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
+  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
   return TAMI_OK;
 }
 
@@ -570,7 +558,7 @@ int tami_forward_backward_workspace(const tami_diagram* d, int64_t n_samples, in
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
   const int grid = bwd_grid(d, n_f, n_samples, nullptr, true);
-  *bytes = kBwStatusBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
+  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
   return TAMI_OK;
 }
 
@@ -589,17 +577,15 @@ int tami_backward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed,
   bool generic_ok = true;
   const int grid = bwd_grid(d, n_f, n_samples, &smem, false, &generic_ok);
   const std::string generic_why = generic_ok ? std::string() : std::string(tami_last_error());
-  const size_t need = kBwStatusBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
+  const size_t need = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
   if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
   tami_diagram* dm = const_cast<tami_diagram*>(d);
   const int sel = jit_select(dm, kJitKindBwd, n_samples, n_f, generic_ok);
   if (sel < 0) return -sel;
   if (sel == 0 && !generic_ok) { set_error(generic_why); return TAMI_EUNSUPPORTED; }
   cudaStream_t st = (cudaStream_t)stream;
-  int* status = static_cast<int*>(workspace);
-  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kBwStatusBytes);
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kBwHeadBytes);
+  cudaError_t e = cudaSuccess;
   int used_grid = grid;
   if (sel == 1) {
     rc = jit_launch(dm, kJitKindBwd, lat, seed, offset, n_samples, X, n_f, beta, gout, nullptr, per_sample_dX,
@@ -616,16 +602,15 @@ int tami_backward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed,
     P.X = X; P.G = gout; P.n_f = n_f; P.beta = beta;
     P.ps_dX = per_sample_dX; P.ps_grad = per_sample_grads;
     P.saved = saved;
-    P.partial = partial; P.status = status;
+    P.partial = partial;
     P.wait_limit = wait_limit();
     if (saved) bwd_kernel<true, false><<<grid, kBlock, smem, st>>>(P);
     else bwd_kernel<false, false><<<grid, kBlock, smem, st>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "bwd_kernel launch");
   }
-  bwd_finalize_kernel<<<n_f + 1, kFinBlock, 0, st>>>(partial, used_grid, n_f, n_samples, gout, status,
-                                                              dsigma_dX, grad_X_re, grad_params);
-  e = cudaGetLastError();
+  e = launch_after(bwd_finalize_kernel, n_f + 1, kFinBlock, st, partial, used_grid, n_f, n_samples, gout, dsigma_dX,
+                   grad_X_re, grad_params);
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "bwd finalize launch");
   });
 }
@@ -645,7 +630,7 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
   bool generic_ok = true;
   const int grid = bwd_grid(d, n_f, n_samples, &smem, true, &generic_ok);
   const std::string generic_why = generic_ok ? std::string() : std::string(tami_last_error());
-  const size_t need = kBwStatusBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
+  const size_t need = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
   if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
   // the diagram's specialised kernel (compiled once and cached with it) or the generic one
   tami_diagram* dm = const_cast<tami_diagram*>(d);
@@ -653,10 +638,8 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
   if (sel < 0) return -sel;
   if (sel == 0 && !generic_ok) { set_error(generic_why); return TAMI_EUNSUPPORTED; }
   cudaStream_t st = (cudaStream_t)stream;
-  int* status = static_cast<int*>(workspace);
-  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kBwStatusBytes);
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kBwHeadBytes);
+  cudaError_t e = cudaSuccess;
   int used_grid = grid;
   if (sel == 1) {
     rc = jit_launch(dm, kJitKindFused, lat, seed, offset, n_samples, X, n_f, beta, gout, per_sample, per_sample_dX,
@@ -672,15 +655,14 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
     P.seed = seed; P.offset = offset; P.n = n_samples;
     P.X = X; P.G = gout; P.n_f = n_f; P.beta = beta;
     P.ps_dX = per_sample_dX; P.ps_grad = per_sample_grads; P.ps_v = per_sample;
-    P.partial = partial; P.status = status;
+    P.partial = partial;
     P.wait_limit = wait_limit();
     bwd_kernel<false, true><<<grid, kBlock, smem, st>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
   }
-  fused_finalize_kernel<<<n_f + 1, kFinBlock, 0, st>>>(partial, used_grid, n_f, n_samples, gout, status, mean, var,
-                                                       dsigma_dX, grad_X_re, grad_params);
-  e = cudaGetLastError();
+  e = launch_after(fused_finalize_kernel, n_f + 1, kFinBlock, st, partial, used_grid, n_f, n_samples, gout, mean, var,
+                   dsigma_dX, grad_X_re, grad_params);
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "fused finalize launch");
   });
 }

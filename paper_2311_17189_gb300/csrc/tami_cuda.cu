@@ -45,7 +45,6 @@ struct FwdParams {
   double* per_sample;           // [n_f][n][2] or null
   double* saved;                // [n_rep + 2 n_rep_ext][n] for the adjoint, or null (momentum mode)
   double* partial;              // [gridDim][n_f][4] or null
-  int* status;                  // device status word or null
   int ring_chunk;               // streamed program: ops per ring buffer (even); 0 when resident
   long long wait_limit;         // bound of the first stage of every mbarrier wait
 };
@@ -64,13 +63,21 @@ __host__ __device__ __forceinline__ size_t fwd_smem_bytes(const TableHeader& h, 
          sizeof(double) * ((2 * (size_t)h.n_xk + 2 * (size_t)h.n_cden) * n_f + (size_t)(h.n_cden + h.n_g2 + 4) * kBlock);
 }
 
+// A block whose staging failed or came late leaves NaN partial sums, and with them NaN means: no
+// status word in global memory, so no launch to clear one before each call.
 template <bool ENERGY_IN, bool SAVE, bool STREAM>
 __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) unsigned long long ring_bar[2];
   const TableHeader& H = P.h;
   const int tid = threadIdx.x;
-  if (!stage_table(smem, P.table, STREAM ? H.off_ops : H.off_opsb, P.status, P.wait_limit)) return;
+  let_next_kernel_start();
+  __shared__ int s_late;                     // set when a bounded wait of this block ran out
+  if (tid == 0) s_late = 0;
+  if (!stage_table(smem, P.table, STREAM ? H.off_ops : H.off_opsb, &s_late, P.wait_limit)) {
+    if (P.partial) nan_row(P.partial + (size_t)blockIdx.x * P.n_f * 4, 4 * P.n_f);
+    return;
+  }
   OpRing R;
   if (STREAM) {
     mbar_init(&ring_bar[0]);
@@ -78,7 +85,7 @@ __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
     R.src = P.table + H.off_ops;
     R.buf = reinterpret_cast<int2*>(smem + H.off_ops);
     R.bar = ring_bar;
-    R.status = P.status;
+    R.status = &s_late;
     R.limit = P.wait_limit;
     R.n_ops = H.n_ops;
     R.chunk = P.ring_chunk;
@@ -108,13 +115,16 @@ __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x)
     fwd_tile<ENERGY_IN, SAVE, STREAM>(H, T, A, tile, Xs, AXI, AXI2, xr_zero, CB, W, M, acc, R);
   if (!P.partial) return;
-  block_reduce_store(M, P.n_f, acc, red, P.partial + (size_t)blockIdx.x * P.n_f * 4);
+  double* row = P.partial + (size_t)blockIdx.x * P.n_f * 4;
+  block_reduce_store(M, P.n_f, acc, red, row);
+  if (s_late) nan_row(row, 4 * P.n_f);
 }
 
 // mean and unbiased variances from per-block partials, summed in block order
 // One block of kFinBlock threads per frequency: the sums over the per-block partials.
 __global__ void __launch_bounds__(kFinBlock) finalize_kernel(const double* partial, int n_blocks, int n_f, long long n,
-                                                            const int* status, double* mean, double* var) {
+                                                            double* mean, double* var) {
+  wait_for_previous_kernel();
   __shared__ double sh[4][kFinBlock];
   const int f = blockIdx.x;
   double s[4] = {0.0, 0.0, 0.0, 0.0};
@@ -129,7 +139,6 @@ __global__ void __launch_bounds__(kFinBlock) finalize_kernel(const double* parti
   double mr = s1r / nn, mi = s1i / nn;
   double vr = n > 1 ? (s2r - s1r * mr) / (nn - 1.0) : 0.0;
   double vi = n > 1 ? (s2i - s1i * mi) / (nn - 1.0) : 0.0;
-  if (status && *status != 0) mr = mi = vr = vi = __longlong_as_double(0x7ff8000000000000ll);
   mean[2 * f] = mr;
   mean[2 * f + 1] = mi;
   if (var) { var[2 * f] = vr; var[2 * f + 1] = vi; }
@@ -245,12 +254,8 @@ bool fwd_staging(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem) 
 }
 
 template <bool E_IN, bool SAVE, bool STREAM>
-int fwd_blocks_per_sm(size_t smem) {
-  cudaFuncSetAttribute(fwd_kernel<E_IN, SAVE, STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_kernel<E_IN, SAVE, STREAM>, kBlock, smem) != cudaSuccess)
-    per_sm = 1;
-  return per_sm < 1 ? 1 : per_sm;
+int fwd_blocks_per_sm(int dev, size_t smem) {
+  return resident_blocks(dev, (const void*)fwd_kernel<E_IN, SAVE, STREAM>, kBlock, smem);
 }
 
 template <bool E_IN, bool SAVE>
@@ -260,7 +265,7 @@ int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max
   if (!fwd_staging(d, P.n_f, &chunk, &smem)) return TAMI_EUNSUPPORTED;
   P.ring_chunk = chunk;
   DeviceProps dp = device_props(d->device);
-  const int per_sm = chunk ? fwd_blocks_per_sm<E_IN, SAVE, true>(smem) : fwd_blocks_per_sm<E_IN, SAVE, false>(smem);
+  const int per_sm = chunk ? fwd_blocks_per_sm<E_IN, SAVE, true>(d->device, smem) : fwd_blocks_per_sm<E_IN, SAVE, false>(d->device, smem);
   long long tiles = (P.n + kBlock - 1) / kBlock;
   long long grid = (long long)dp.sms * per_sm;
   if (grid > tiles) grid = tiles;
@@ -287,8 +292,8 @@ int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nul
     return (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
   }
   // the saving instance shares the grid (one workspace size for both)
-  const int per_sm = chunk ? std::min(fwd_blocks_per_sm<false, false, true>(smem), fwd_blocks_per_sm<false, true, true>(smem))
-                           : std::min(fwd_blocks_per_sm<false, false, false>(smem), fwd_blocks_per_sm<false, true, false>(smem));
+  const int per_sm = chunk ? std::min(fwd_blocks_per_sm<false, false, true>(d->device, smem), fwd_blocks_per_sm<false, true, true>(d->device, smem))
+                           : std::min(fwd_blocks_per_sm<false, false, false>(d->device, smem), fwd_blocks_per_sm<false, true, false>(d->device, smem));
   long long tiles = (n + kBlock - 1) / kBlock;
   long long grid = (long long)dp.sms * per_sm;
   if (grid > tiles) grid = tiles;
@@ -327,14 +332,13 @@ FwdParams make_params(const tami_diagram* d, int n_f, double beta) {
   return P;
 }
 
-constexpr size_t kStatusBytes = 256;
+constexpr size_t kHeadBytes = 256;   // the partial sums start here in a workspace
 
 std::atomic<int> g_staging_mode{TAMI_STAGING_AUTO};
 std::atomic<int> g_ring_chunk{512};
 std::atomic<long long> g_wait_limit{kSpinLimit};
 
-// Scratch of tami_forward_noalloc: a status word (first 256 bytes) followed by the per-block
-// partial sums [grid][n_f][4].  It lives in the library image, so every GPU that loads the
+// Scratch of tami_forward_noalloc: the per-block partial sums [grid][n_f][4] after kHeadBytes.  It lives in the library image, so every GPU that loads the
 // library holds these bytes until the process exits; no call allocates them.
 constexpr size_t kNoAllocScratchBytes = 4u << 20;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -456,7 +460,7 @@ int tami_forward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, si
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
   int grid = grid_for(d, n_f, n_samples);
-  *bytes = kStatusBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
+  *bytes = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
   return TAMI_OK;
 }
 
@@ -473,16 +477,13 @@ int tami_forward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed, 
   if (((uintptr_t)workspace & 255) != 0) { set_error("workspace must be 256-byte aligned"); return TAMI_EINVAL; }
   bool generic_ok = true;
   const int grid = grid_for(d, n_f, n_samples, &generic_ok);
-  const size_t need = kStatusBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
+  const size_t need = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
   if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
   tami_diagram* dm = const_cast<tami_diagram*>(d);
   const int sel = jit_select(dm, kJitKindFwd, n_samples, n_f, generic_ok);
   if (sel < 0) return -sel;
   cudaStream_t st = (cudaStream_t)stream;
-  int* status = static_cast<int*>(workspace);
-  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kStatusBytes);
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  double* partial = reinterpret_cast<double*>(static_cast<char*>(workspace) + kHeadBytes);
   int used_grid = grid;
   if (sel == 1) {
     rc = jit_launch(dm, kJitKindFwd, lat, seed, offset, n_samples, X, n_f, beta, nullptr, per_sample, nullptr,
@@ -497,12 +498,10 @@ int tami_forward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed, 
     P.per_sample = per_sample;
     P.saved = saved;
     P.partial = partial;
-    P.status = status;
     rc = saved ? launch_fwd<false, true>(d, P, st, grid) : launch_fwd<false, false>(d, P, st, grid);
     if (rc) return rc;
   }
-  finalize_kernel<<<n_f, kFinBlock, 0, st>>>(partial, used_grid, n_f, n_samples, status, mean, var);
-  e = cudaGetLastError();
+  const cudaError_t e = launch_after(finalize_kernel, n_f, kFinBlock, st, partial, used_grid, n_f, n_samples, mean, var);
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "finalize launch");
   });
 }
@@ -522,7 +521,7 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
   bool generic_ok = true;
   const int grid = grid_for(d, n_f, n_samples, &generic_ok);
   if (!generic_ok) return TAMI_EUNSUPPORTED;   // this call runs the generic kernel only
-  const size_t need = kStatusBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
+  const size_t need = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
   if (need > kNoAllocScratchBytes) {
     set_error("tami_forward_noalloc: needs " + std::to_string(need) + " bytes of scratch for n_f=" +
               std::to_string(n_f) + " over " + std::to_string(grid) + " blocks, above the fixed " +
@@ -532,23 +531,18 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
   unsigned char* base = noalloc_scratch(d->device);
   if (!base) return TAMI_ECUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  int* status = reinterpret_cast<int*>(base);
-  double* partial = reinterpret_cast<double*>(base + kStatusBytes);
-  // the status word must start at zero; the partials are fully rewritten by every launch
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(int), st);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+  double* partial = reinterpret_cast<double*>(base + kHeadBytes);
+  // the partials are fully rewritten by every launch
   FwdParams P = make_params(d, n_f, beta);
   P.t = lat->t; P.tp = lat->tp; P.mu = lat->mu; P.kx = lat->kx_ext; P.ky = lat->ky_ext;
   P.seed = seed; P.offset = offset; P.n = n_samples;
   P.X = X;
   P.per_sample = per_sample;
   P.partial = partial;
-  P.status = status;
   jit_mark_generic(const_cast<tami_diagram*>(d));
   rc = launch_fwd<false, false>(d, P, st, grid);
   if (rc) return rc;
-  finalize_kernel<<<n_f, kFinBlock, 0, st>>>(partial, grid, n_f, n_samples, status, mean, var);
-  e = cudaGetLastError();
+  const cudaError_t e = launch_after(finalize_kernel, n_f, kFinBlock, st, partial, grid, n_f, n_samples, mean, var);
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "finalize launch");
   });
 }

@@ -7,6 +7,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <vector>
 
 #include "tami_internal.h"
 #include "tami_devmath.cuh"
@@ -41,7 +42,8 @@ __host__ __device__ __forceinline__ int align16(int b) { return (b + 15) & ~15; 
 // into shared memory, completed on the mbarrier `bar` (initialised once with count 1 by
 // mbar_init).  `parity` is the phase being completed: 0 for the first use, then alternating.
 // The caller must __syncthreads() before a re-fill so that no thread still reads the old data.
-// Every wait is bounded; on timeout the status word is set and the copy is waited for again.
+// Every wait is bounded; on timeout the status word (a block's own, in shared memory, or a plan's) is
+// set and the copy is waited for again.
 __device__ __forceinline__ void mbar_init(unsigned long long* bar) {
   if (threadIdx.x == 0) {
     const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
@@ -111,6 +113,17 @@ __device__ __forceinline__ bool stage_table(unsigned char* dst, const unsigned c
   return !__syncthreads_or(!ok);
 }
 
+// the block's threads fill a row of partial sums with NaN
+__device__ __forceinline__ void nan_row(double* row, int n) {
+  for (int i = threadIdx.x; i < n; i += kBlock) row[i] = __longlong_as_double(0x7ff8000000000000ll);
+}
+
+// Start of a kernel launched by launch_after: waits until the stream's previous kernel has ended
+// and its writes are visible.
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// In the kernel before it: the next kernel's blocks may be brought in while this one still runs.
+__device__ __forceinline__ void let_next_kernel_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 // ------------------------------------------------------------------------------- host helpers
 inline int cuda_fail(cudaError_t e, const char* what) {
   set_error(std::string(what) + ": " + cudaGetErrorString(e));
@@ -131,6 +144,48 @@ inline DeviceProps device_props(int dev) {
     }
   }
   return cache[dev];
+}
+
+// Resident blocks per SM of one of the library's kernels at `block` threads and `smem` bytes of
+// dynamic shared memory (at least 1), its shared-memory limit raised as needed.  The two runtime
+// queries take several microseconds, as long as a small launch, and every call asks for the same
+// few combinations: the answers are kept per device, kernel, block and size (a table of at most
+// kMost entries; the kernels are the library's own, so their addresses stay).
+inline int resident_blocks(int dev, const void* kernel, int block, size_t smem) {
+  struct Known { int dev; const void* kernel; int block; size_t smem; int per_sm; };
+  constexpr size_t kMost = 256;
+  static std::mutex mu;
+  static std::vector<Known> known;
+  std::lock_guard<std::mutex> lk(mu);
+  size_t limit = 0;
+  for (const Known& k : known)
+    if (k.dev == dev && k.kernel == kernel) {
+      if (k.block == block && k.smem == smem) return k.per_sm;
+      if (k.smem > limit) limit = k.smem;
+    }
+  // the limit only grows: a smaller one set for one call would fail another thread's launch
+  if (smem > limit || limit == 0) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess) per_sm = 1;
+  if (per_sm < 1) per_sm = 1;
+  if (known.size() < kMost) known.push_back({dev, kernel, block, smem, per_sm});
+  return per_sm;
+}
+
+// Launches `kernel` so that its launch overlaps the end of the stream's previous kernel
+// (programmatic dependent launch); the kernel begins with wait_for_previous_kernel().
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = st;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
 }  // namespace dev

@@ -1100,11 +1100,12 @@ int jit_select(tami_diagram* d, int kind, int64_t n, int n_f, bool generic_ok) {
   // large enough to repay a compilation: 2^21 Monte Carlo samples, or 2^25 (row, frequency) values;
   // a table the generic kernel cannot take goes to the specialised one at any size
   const bool big = !generic_ok || (kind == kKindEnergy ? (double)n * n_f >= 33554432.0 : n >= (int64_t(1) << 21));
+  if (mode == TAMI_JIT_AUTO && !big) return 0;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, d->device);
   const bool fits = (kind == kKindEnergy || n_f <= kJitMaxFreq) &&
                     jit_smem(d->hdr, kind, n_f, lockstep_block(d->hdr, kind)) <= (size_t)optin;
-  if (mode == TAMI_JIT_AUTO && (!big || !fits || !jit_supported(d->hdr, kind, nullptr))) return 0;
+  if (mode == TAMI_JIT_AUTO && (!fits || !jit_supported(d->hdr, kind, nullptr))) return 0;
   if (!fits) { set_error("specialised kernel: frequencies beyond its per-thread sums or shared memory"); return -TAMI_EUNSUPPORTED; }
   const int rc = jit_prepare(d, kind);
   if (rc == TAMI_OK) return 1;
