@@ -120,6 +120,69 @@ __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
   if (s_late) nan_row(row, 4 * P.n_f);
 }
 
+// Shared memory of coop_kernel: table | Xs | AXI, AXI2 | the tile's buffers
+__host__ __device__ __forceinline__ size_t coop_smem_bytes(const TableHeader& h, int n_f, int ring_chunk) {
+  return fwd_table_smem(h, ring_chunk) + sizeof(double) * ((2 * (size_t)h.n_xk + 2 * (size_t)h.n_cden) * n_f +
+                                                (size_t)coop_rows(h) * kCoopSamples);
+}
+
+template <bool ENERGY_IN, bool SAVE, bool STREAM>
+__global__ void __launch_bounds__(kBlock) coop_kernel(const FwdParams P) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long ring_bar[2];
+  const TableHeader& H = P.h;
+  let_next_kernel_start();
+  __shared__ int s_late;                     // set when a bounded wait of this block ran out
+  if (threadIdx.x == 0) s_late = 0;
+  if (!stage_table(smem, P.table, STREAM ? H.off_ops : H.off_opsb, &s_late, P.wait_limit)) {
+    if (P.partial) nan_row(P.partial + (size_t)blockIdx.x * P.n_f * 4, 4 * P.n_f);
+    return;
+  }
+  OpRing R;
+  if (STREAM) {
+    mbar_init(&ring_bar[0]);
+    mbar_init(&ring_bar[1]);
+    R.src = P.table + H.off_ops;
+    R.buf = reinterpret_cast<int2*>(smem + H.off_ops);
+    R.bar = ring_bar;
+    R.status = &s_late;
+    R.limit = P.wait_limit;
+    R.n_ops = H.n_ops;
+    R.chunk = P.ring_chunk;
+    R.n_chunks = (H.n_ops + P.ring_chunk - 1) / P.ring_chunk;
+    R.waits[0] = R.waits[1] = 0;
+    R.failed = false;
+  }
+  double* Xs = reinterpret_cast<double*>(smem + fwd_table_smem(H, STREAM ? P.ring_chunk : 0));
+  double* AXI = Xs + 2 * H.n_xk * P.n_f;
+  double* AXI2 = AXI + H.n_cden * P.n_f;
+  const CoopBuffers B = coop_buffers(H, AXI2 + H.n_cden * P.n_f);
+  const TableView T = table_view(smem, H);
+  stage_freqs(H, T, P.X, P.n_f, Xs);
+  double acc[ENERGY_IN ? 1 : kCoopFreqPerThread][4];
+  const int w = threadIdx.x / kCoopSamples, sl = threadIdx.x % kCoopSamples;
+  if (!ENERGY_IN)
+    for (int f = w, i = 0; f < P.n_f; f += kCoopWarps, ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0;
+  __syncthreads();
+  const bool xr_zero = freq_constants(H, T, Xs, P.n_f, AXI, AXI2);
+  TileArgs A;
+  A.t = P.t; A.tp = P.tp; A.mu = P.mu; A.kx = P.kx; A.ky = P.ky; A.beta = P.beta;
+  A.seed = P.seed; A.offset = P.offset; A.n = P.n; A.E_in = P.E_in; A.per_sample = P.per_sample;
+  A.saved = P.saved;
+  A.n_f = P.n_f;
+  const long long n_tiles = (P.n + kCoopSamples - 1) / kCoopSamples;
+  for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x)
+    coop_tile<ENERGY_IN, SAVE, STREAM>(H, T, A, tile, Xs, AXI, AXI2, xr_zero, B, acc, R);
+  if (ENERGY_IN) return;
+  double* row = P.partial + (size_t)blockIdx.x * P.n_f * 4;
+  for (int f = w, i = 0; f < P.n_f; f += kCoopWarps, ++i)
+    for (int k = 0; k < 4; ++k) {
+      double v = acc[i][k];
+      for (int off = kCoopSamples / 2; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+      if (sl == 0) row[4 * f + k] = s_late ? __longlong_as_double(0x7ff8000000000000ll) : v;
+    }
+}
+
 // mean and unbiased variances from per-block partials, summed in block order
 // One block of kFinBlock threads per frequency: the sums over the per-block partials.
 __global__ void __launch_bounds__(kFinBlock) finalize_kernel(const double* partial, int n_blocks, int n_f, long long n,
@@ -258,10 +321,45 @@ int fwd_blocks_per_sm(int dev, size_t smem) {
   return resident_blocks(dev, (const void*)fwd_kernel<E_IN, SAVE, STREAM>, kBlock, smem);
 }
 
+// How a launch that takes the tile of few samples (coop_tile) stages its table, as fwd_staging; false
+// where it does not take it.  Monte Carlo launches take it up to two 128-sample tiles per SM, where
+// those leave SMs idle and the tile's latency is the launch's: order 4, 16 frequencies, 5000 samples
+// 114 -> 53 us; order 3, 32 frequencies with per-sample values, 20 000 samples 86 -> 74 us, but
+// 65 537 samples 121 -> 148 us.  Energy input, which keeps no running sums, takes it at every size
+// (order 4, 10 000 rows x 30 frequencies 156 -> 64 us; the evaluation example, 100 000 x 50, 103 -> 62
+// us; order 3, 300 000 x 100, 908 -> 755 us; two external frequencies, 250 000 x 100, 3.41 -> 3.02 ms).
+// Above kCoopMaxFreq frequencies a thread's running sums would not fit.
+bool coop_staging(const tami_diagram* d, int n_f, long long n, bool energy_in, int* ring_chunk, size_t* smem) {
+  if (n_f > kCoopMaxFreq || (!energy_in && n > 2LL * kBlock * device_props(d->device).sms)) return false;
+  const size_t optin = device_props(d->device).smem_optin;
+  *ring_chunk = staging_mode() != TAMI_STAGING_STREAMED && coop_smem_bytes(d->hdr, n_f, 0) <= optin ? 0 : ring_chunk_ops();
+  *smem = coop_smem_bytes(d->hdr, n_f, *ring_chunk);
+  return *smem <= optin;
+}
+
+template <bool E_IN, bool SAVE>
+int coop_blocks_per_sm(int dev, int chunk, size_t smem) {
+  return resident_blocks(dev, chunk ? (const void*)coop_kernel<E_IN, SAVE, true> : (const void*)coop_kernel<E_IN, SAVE, false>,
+                         kBlock, smem);
+}
+
+template <bool E_IN, bool SAVE>
+int launch_coop(const tami_diagram* d, FwdParams& P, int chunk, size_t smem, cudaStream_t stream, int max_blocks) {
+  P.ring_chunk = chunk;
+  const long long tiles = (P.n + kCoopSamples - 1) / kCoopSamples;
+  long long grid = std::min(tiles, (long long)device_props(d->device).sms * coop_blocks_per_sm<E_IN, SAVE>(d->device, chunk, smem));
+  if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
+  if (chunk) coop_kernel<E_IN, SAVE, true><<<(unsigned)grid, kBlock, smem, stream>>>(P);
+  else coop_kernel<E_IN, SAVE, false><<<(unsigned)grid, kBlock, smem, stream>>>(P);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "coop_kernel launch");
+}
+
 template <bool E_IN, bool SAVE>
 int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max_blocks) {
   size_t smem = 0;
   int chunk = 0;
+  if (coop_staging(d, P.n_f, P.n, E_IN, &chunk, &smem)) return launch_coop<E_IN, SAVE>(d, P, chunk, smem, stream, max_blocks);
   if (!fwd_staging(d, P.n_f, &chunk, &smem)) return TAMI_EUNSUPPORTED;
   P.ring_chunk = chunk;
   DeviceProps dp = device_props(d->device);
@@ -281,7 +379,7 @@ int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max
 // Grid of a momentum-mode forward launch (the workspace holds one partial row per block).  When
 // the generic kernel cannot stage the table (*generic_ok = false) only the specialised kernel can
 // run it, whose launch is clamped to the rows of the workspace: 4 blocks per SM.
-int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nullptr) {
+int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nullptr, bool coop = true) {
   DeviceProps dp = device_props(d->device);
   size_t smem = 0;
   int chunk = 0;
@@ -290,6 +388,15 @@ int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nul
   if (!ok) {
     const long long tiles = (n + kBlock - 1) / kBlock;
     return (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
+  }
+  {
+    size_t cs = 0;
+    int cc = 0;
+    if (coop && coop_staging(d, n_f, n, false, &cc, &cs)) {
+      const int per_sm = std::min(coop_blocks_per_sm<false, false>(d->device, cc, cs),
+                                  coop_blocks_per_sm<false, true>(d->device, cc, cs));
+      return (int)std::min((n + kCoopSamples - 1) / kCoopSamples, (long long)dp.sms * per_sm);
+    }
   }
   // the saving instance shares the grid (one workspace size for both)
   const int per_sm = chunk ? std::min(fwd_blocks_per_sm<false, false, true>(d->device, smem), fwd_blocks_per_sm<false, true, true>(d->device, smem))
@@ -519,7 +626,7 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
   if (!lat || !X || !mean || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
   if (!beta_ok(beta)) return TAMI_EINVAL;
   bool generic_ok = true;
-  const int grid = grid_for(d, n_f, n_samples, &generic_ok);
+  int grid = grid_for(d, n_f, n_samples, &generic_ok, false);
   if (!generic_ok) return TAMI_EUNSUPPORTED;   // this call runs the generic kernel only
   const size_t need = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
   if (need > kNoAllocScratchBytes) {
@@ -528,6 +635,7 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
               std::to_string(kNoAllocScratchBytes) + "-byte array; use tami_forward with a workspace");
     return TAMI_EINVAL;
   }
+  grid = std::min(grid_for(d, n_f, n_samples), (int)((kNoAllocScratchBytes - kHeadBytes) / (sizeof(double) * 4 * (size_t)n_f)));
   unsigned char* base = noalloc_scratch(d->device);
   if (!base) return TAMI_ECUDA;
   cudaStream_t st = (cudaStream_t)stream;

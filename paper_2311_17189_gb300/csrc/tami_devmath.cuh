@@ -779,10 +779,11 @@ __device__ __forceinline__ double dag_step(double F, double a, double v, int fir
 // the Bose-type segments (sigma = -1) take 1 - y = -(e^t - 1) from the same exponential.  With
 // DUAL, fvd holds each value's derivative with respect to its own argument (order k + 1).
 // seg = {combo, sigma, v_begin, first v with k >= 1, v_end}; fvr[v] = {sign, k}.
-template <bool BOSE, bool DUAL>
+// S: the stride of x and fv (1, or the samples of a tile where they lie in shared memory).
+template <bool BOSE, bool DUAL, int S = 1>
 __device__ __forceinline__ void fermi_segment(const int* seg, const int* fvr, const double* x, double beta,
                                               double* fv, double* fvd) {
-  const double xv = x[seg[0]];
+  const double xv = x[seg[0] * S];
   double em = 0.0;
   const double y = exp_neg<BOSE>(neg_bits(imul(beta, fabs(xv))), em);
   const double rD = rcp(BOSE ? neg_bits(em) : 1.0 + y);
@@ -792,14 +793,14 @@ __device__ __forceinline__ void fermi_segment(const int* seg, const int* fvr, co
   double d1 = 0.0;
   if (DUAL) d1 = neg_bits(imul(beta, imul(g, h)));
   for (int v = seg[2]; v < seg[3]; ++v) {
-    fv[v] = fvr[2 * v] > 0 ? g : h;
+    fv[v * S] = fvr[2 * v] > 0 ? g : h;
     if (DUAL) fvd[v] = d1;
   }
   for (int v = seg[3]; v < seg[4]; ++v) {
     const bool pos = fvr[2 * v] > 0;
     const int k = fvr[2 * v + 1];
     const double gg = pos ? g : h, hg = pos ? h : g;
-    fv[v] = fermi_poly(k, gg, hg, beta);
+    fv[v * S] = fermi_poly(k, gg, hg, beta);
     if (DUAL) fvd[v] = fermi_poly(k + 1, gg, hg, beta);
   }
 }

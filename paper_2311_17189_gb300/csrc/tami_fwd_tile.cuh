@@ -127,8 +127,8 @@ struct OpRing {
 // Sum over a group's terms of A_t prod FT factors, by the group's pole-tree program: one step per
 // edge of the (shared-sub-sum) tree, v[dst] = F * (leaf ? A[ref] : v[ref]) + (first ? 0 : v[dst]),
 // over value slots; the root's sum is written by the group's last op.  Both operand loads use
-// in-range indices, the select picks one.  STREAM: the ops come from the ring.
-template <bool STREAM>
+// in-range indices, the select picks one.  S: the stride of fv.  STREAM: the ops come from the ring.
+template <bool STREAM, int S = 1>
 __device__ __forceinline__ double pole_tree(const TableView& T, OpRing& R, int op0, int op1, const double* fv) {
   double v[kMaxSlots];
   v[0] = 0.0;
@@ -139,7 +139,7 @@ __device__ __forceinline__ double pole_tree(const TableView& T, OpRing& R, int o
     const int ref = op.x >> kOpRefShift;
     const bool leaf = op.x & kOpLeaf;
     const double a = T.leafA[leaf ? ref : 0], b = v[leaf ? 0 : ref];
-    v[dst] = dag_step(fv[op.y], leaf ? a : b, v[dst], op.x & kOpFirst);
+    v[dst] = dag_step(fv[op.y * S], leaf ? a : b, v[dst], op.x & kOpFirst);
   }
   return v[dst];
 }
@@ -254,14 +254,15 @@ __device__ __forceinline__ bool freq_constants(const TableHeader& H, const Table
 // first (g2_const).  The products run on the integer pipes (imul, the FP64 unit's bits), beside the
 // sums' fmas (two external frequencies, 250 000 rows x 100: 4.25 -> 3.37 ms; order-4 forward, 10^6
 // samples x 21 frequencies: 2.82 -> 2.50 ms).
-template <bool XR_ZERO>
+// S: the samples of a tile (the stride of CB and W).
+template <bool XR_ZERO, int S>
 __device__ __forceinline__ void phase2_sample(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
                                               int f, const double* Xs, const double* AXI, const double* AXI2,
                                               const double* CB, const double* W, double& vr_out, double& vi_out) {
   // values: [0, n_cden) the reciprocals 1/D_c, then the product nodes
   double vre[kMaxCplxDens + kMaxProdNodes], vim[kMaxCplxDens + kMaxProdNodes];
   for (int c = 0; c < H.n_cden; ++c) {
-    const double b = CB[c * kBlock + sl];
+    const double b = CB[c * S + sl];
     // D = g_c Y_{k_c f} + b
     const double Dr = XR_ZERO ? b : fma(T.cden_a[c], Xs[2 * (T.cden_xk[c] * A.n_f + f)], b);
     const double r = rcp(fma(Dr, Dr, AXI2[c * A.n_f + f]));
@@ -276,7 +277,7 @@ __device__ __forceinline__ void phase2_sample(const TableHeader& H, const TableV
   }
   double vr = H.g2_const ? W[sl] : 0.0, vi = 0.0;
   for (int hg = H.g2_const; hg < H.n_g2; ++hg) {
-    const double w = W[hg * kBlock + sl];
+    const double w = W[hg * S + sl];
     const int v = T.g2node[hg];
     vr = fma(w, vre[v], vr);
     vi = fma(w, vim[v], vi);
@@ -439,8 +440,8 @@ __device__ __forceinline__ void phase2_loop(const TableHeader& H, const TableVie
       const int pa = M.p0 + j, pb = pa + 1;
       const int fa = pa / kBlock, sla = pa % kBlock, fb = pb / kBlock, slb = pb % kBlock;
       double ar, ai, br, bi;
-      phase2_sample<XR_ZERO>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
-      phase2_sample<XR_ZERO>(H, T, A, slb, fb, Xs, AXI, AXI2, CB, W, br, bi);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, slb, fb, Xs, AXI, AXI2, CB, W, br, bi);
       const bool sa = sla == 0 && j > 0, sb = slb == 0;
       swap_sums(sa, cur, oth);
       crossed |= sa;
@@ -452,7 +453,7 @@ __device__ __forceinline__ void phase2_loop(const TableHeader& H, const TableVie
     if (j < A.n_f) {
       const int pa = M.p0 + j, fa = pa / kBlock, sla = pa % kBlock;
       double ar, ai;
-      phase2_sample<XR_ZERO>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
       const bool sa = sla == 0 && j > 0;
       swap_sums(sa, cur, oth);
       crossed |= sa;
@@ -468,17 +469,161 @@ __device__ __forceinline__ void phase2_loop(const TableHeader& H, const TableVie
     const int se = fi ? M.se1 : M.se0;
     for (; sl + M.sstep < se && s0 + sl + M.sstep < A.n; sl += 2 * M.sstep) {
       double ar, ai, br, bi;
-      phase2_sample<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
-      phase2_sample<XR_ZERO>(H, T, A, sl + M.sstep, f, Xs, AXI, AXI2, CB, W, br, bi);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl + M.sstep, f, Xs, AXI, AXI2, CB, W, br, bi);
       phase2_store(A, f, s0 + sl, ar, ai, acc[fi]);
       phase2_store(A, f, s0 + sl + M.sstep, br, bi, acc[fi]);
     }
     for (; sl < se && s0 + sl < A.n; sl += M.sstep) {
       double ar, ai;
-      phase2_sample<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
+      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
       phase2_store(A, f, s0 + sl, ar, ai, acc[fi]);
     }
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The tile of few samples: the block's four warps share the phase-1 work of 32 samples (lane =
+// sample), warp w taking the momenta, lines, combinations, segments and groups w, w + 4, ..., with
+// every per-sample quantity in shared memory, [index][32]; in phase 2 warp w takes the frequencies
+// w, w + 4, ....  A launch of few samples then reaches four times as many SMs and its tile's latency,
+// a serial walk over the table, shrinks with the walk.
+constexpr int kCoopSamples = 32;
+constexpr int kCoopWarps = kBlock / kCoopSamples;
+constexpr int kCoopMaxFreq = 256;
+constexpr int kCoopFreqPerThread = kCoopMaxFreq / kCoopWarps;
+
+template <bool V>
+struct BoolConst { static constexpr bool value = V; };
+
+struct CoopBuffers {   // each [count][kCoopSamples]
+  double *K, *E, *x, *fv, *rr, *W1, *W, *CB;
+};
+__host__ __device__ __forceinline__ int coop_rows(const TableHeader& h) {
+  return 2 * h.m + h.N + h.n_combo + h.n_fv + h.n_rden + h.n_g1 + h.n_g2 + h.n_cden;
+}
+__device__ __forceinline__ CoopBuffers coop_buffers(const TableHeader& H, double* p) {
+  CoopBuffers B;
+  auto take = [&](int rows) { double* q = p; p += rows * kCoopSamples; return q; };
+  B.K = take(2 * H.m); B.E = take(H.N); B.x = take(H.n_combo); B.fv = take(H.n_fv); B.rr = take(H.n_rden);
+  B.W1 = take(H.n_g1); B.W = take(H.n_g2); B.CB = take(H.n_cden);
+  return B;
+}
+
+// Same operations in the same order as fwd_tile, so the same per-sample bits.  STREAM: the program
+// comes through the ring R; a warp steps over the ops of the other warps' groups, since every thread
+// of the block takes part in every move to the next chunk.  Ends with a barrier.
+template <bool ENERGY_IN, bool SAVE, bool STREAM>
+__device__ __forceinline__ void coop_tile(const TableHeader& H, const TableView& T, const TileArgs& A, long long tile,
+                                          const double* Xs, const double* AXI, const double* AXI2, bool xr_zero,
+                                          const CoopBuffers& B, double (*acc)[4], OpRing& R) {
+  constexpr int S = kCoopSamples;
+  if (STREAM) R.begin();
+  const int w = threadIdx.x / S, sl = threadIdx.x % S;
+  const long long s = tile * S + sl;
+  const bool active = s < A.n;
+  const long long sc = active ? s : A.n - 1;      // a lane past the end repeats the last sample and writes nothing
+  if (!ENERGY_IN) {
+    const unsigned long long sg = A.offset + (unsigned long long)sc;
+    for (int l = w; l < H.m; l += kCoopWarps) {
+      uint32_t c[4] = {(uint32_t)sg, (uint32_t)(sg >> 32), (uint32_t)l, 0u};
+      philox4x32_10(c, (uint32_t)A.seed, (uint32_t)(A.seed >> 32));
+      B.K[2 * l * S + sl] = to_momentum(c[0], c[1]);
+      B.K[(2 * l + 1) * S + sl] = to_momentum(c[2], c[3]);
+    }
+    __syncthreads();
+  }
+  for (int r = w; r < H.n_rep; r += kCoopWarps) {
+    const int line = T.repl[r];
+    if (ENERGY_IN) {
+      B.E[line * S + sl] = A.E_in[sc * H.N + line];
+      continue;
+    }
+    double ax = 0.0, ay = 0.0;
+    for (int q = T.lm_ptr[r], q0 = q; q < T.lm_ptr[r + 1]; ++q) {
+      const double cf = T.lm_c[q];
+      const int l = T.lm_l[q];
+      const double kx = l < H.m ? B.K[2 * l * S + sl] : A.kx, ky = l < H.m ? B.K[(2 * l + 1) * S + sl] : A.ky;
+      ax = q == q0 ? coef_mul(cf, kx) : fma(cf, kx, ax);
+      ay = q == q0 ? coef_mul(cf, ky) : fma(cf, ky, ay);
+    }
+    double E;
+    if (SAVE && r < H.n_rep_ext) {
+      double gx, gy;
+      E = line_energy_grad(ax, ay, A.t, A.tp, A.mu, gx, gy);
+      if (active) {
+        A.saved[(size_t)(H.n_rep + 2 * r) * A.n + s] = gx;
+        A.saved[(size_t)(H.n_rep + 2 * r + 1) * A.n + s] = gy;
+      }
+    } else {
+      E = line_energy(ax, ay, A.t, A.tp, A.mu);
+    }
+    B.E[line * S + sl] = E;
+    if (SAVE && active) A.saved[(size_t)r * A.n + s] = E;
+  }
+  __syncthreads();
+  for (int u = w; u < H.n_combo; u += kCoopWarps) {
+    int q = T.combo_ptr[u];
+    const int q1 = T.combo_ptr[u + 1];
+    double v = q < q1 ? coef_mul(T.combo_c[q], B.E[T.combo_j[q] * S + sl]) : 0.0;
+    for (++q; q < q1; ++q) v = fma(T.combo_c[q], B.E[T.combo_j[q] * S + sl], v);
+    B.x[u * S + sl] = v;
+  }
+  __syncthreads();
+  for (int b = w; b < H.n_fseg; b += kCoopWarps) {
+    if (b < H.n_fseg_bose)
+      fermi_segment<true, false, S>(T.fseg + 8 * b, T.fvr, B.x + sl, A.beta, B.fv + sl, nullptr);
+    else
+      fermi_segment<false, false, S>(T.fseg + 8 * b, T.fvr, B.x + sl, A.beta, B.fv + sl, nullptr);
+  }
+  for (int i = w; i < H.n_rden; i += kCoopWarps) B.rr[i * S + sl] = rcp(B.x[T.rden[2 * i] * S + sl]);
+  for (int c = w; c < H.n_cden; c += kCoopWarps) {
+    const double xv = B.x[T.cden[2 * c] * S + sl];
+    B.CB[c * S + sl] = T.cden[2 * c + 1] > 0 ? xv : -xv;
+  }
+  __syncthreads();
+  for (int gi = STREAM ? 0 : w; gi < H.n_g1; gi += STREAM ? 1 : kCoopWarps) {
+    if (STREAM && gi % kCoopWarps != w) {
+      while (T.g1[4 * gi + 1] > R.hi) R.advance();
+      continue;
+    }
+    double ft = pole_tree<STREAM, S>(T, R, T.g1[4 * gi], T.g1[4 * gi + 1], B.fv + sl);
+    for (int q = T.g1[4 * gi + 2]; q < T.g1[4 * gi + 3]; ++q) {
+      const double r = B.rr[T.g1rd[2 * q] * S + sl];
+      for (int pw = T.g1rd[2 * q + 1]; pw > 0; --pw) ft = imul(ft, r);
+    }
+    B.W1[gi * S + sl] = ft;
+  }
+  __syncthreads();
+  // a group's terms come in runs of one target (fwd_tile's order): each target's run by one warp
+  for (int gi = 0; gi < H.n_g1;) {
+    const int tg = T.g1_tgt[gi];
+    int ge = gi + 1;
+    while (ge < H.n_g1 && T.g1_tgt[ge] == tg) ++ge;
+    if (tg % kCoopWarps == w) {
+      double v = 0.0;
+      for (int i = gi; i < ge; ++i) v += B.W1[i * S + sl];
+      B.W[tg * S + sl] = v;
+    }
+    gi = ge;
+  }
+  __syncthreads();
+  auto phase2 = [&](auto zero) {
+    constexpr bool XR_ZERO = decltype(zero)::value;
+    for (int f = w, i = 0; f < A.n_f; f += kCoopWarps, ++i) {
+      double vr, vi;
+      phase2_sample<XR_ZERO, S>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, vr, vi);
+      if (!active) continue;
+      if (ENERGY_IN) {
+        double2* o = reinterpret_cast<double2*>(A.per_sample) + (size_t)f * A.n + s;
+        *o = make_double2(vr, vi);
+      } else {
+        phase2_store(A, f, s, vr, vi, acc[i]);
+      }
+    }
+  };
+  if (xr_zero) phase2(BoolConst<true>{}); else phase2(BoolConst<false>{});
+  __syncthreads();
 }
 
 // Sum the per-thread accumulators of the block in a fixed order into out[n_f][4].
