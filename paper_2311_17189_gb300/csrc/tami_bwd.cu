@@ -47,6 +47,7 @@ struct BwdParams {
   double* ps_v;          // fused pass: [n_f][n][2] each sample's value, or null
   double* partial;       // [grid][2 n_f + 3]
   long long wait_limit;   // bound of the first stage of the staging wait
+  int lq;                // log2 of the lanes that share a sample's frequencies
 };
 
 // Values each block reduces: dv/dX [n_f][2], the three parameter gradients and, in the fused pass,
@@ -73,12 +74,14 @@ __host__ __device__ __forceinline__ size_t bwd_smem_bytes(const TableHeader& h, 
 // group is group 0 (its weight adjoint, sum_f Re g_f, is the same for every sample: the caller
 // sets it from a per-block sum) and the imaginary-axis case is a template parameter.
 template <bool XR_ZERO, bool FWD>
-__device__ __forceinline__ void bwd_phase2(const TableHeader& H, int n_f, long long s, const BwdParams& P,
+__device__ __forceinline__ void bwd_phase2(const TableHeader& H, int n_f, long long s, int q0, bool act, const BwdParams& P,
                                            const double* Xs, const double* Gs, const double* AXI, const double* AXI2,
                                            const double* cden_a, const int* g2, const int* g2cd, const int* pnode,
                                            const int* g2node, const double* pW, const double* b, const double* W2,
                                            double* Wb2, double* bb, double* accX, double* accV) {
-  for (int f = 0; f < n_f; ++f) {
+  // the running sums sit at the lane's own count j of its frequencies, the same in every lane: local
+  // memory is interleaved by thread, and lanes that index it differently touch a line each
+  for (int f = q0, j = 0; f < n_f; f += 1 << P.lq, ++j) {
     const double Xr = Xs[2 * f], gr = Gs[2 * f], gim = Gs[2 * f + 1], ngr = -gr, ngi = -gim;
     double vre[kBwCden + kMaxProdNodes], vim[kBwCden + kMaxProdNodes], U_re[kBwCden], U_im[kBwCden];
     for (int c = 0; c < H.n_cden; ++c) {
@@ -119,17 +122,18 @@ __device__ __forceinline__ void bwd_phase2(const TableHeader& H, int n_f, long l
       dvi = fma(-cden_a[c], Zi, dvi);
       bb[c] = fma(ngr, Zr, fma(ngi, Zi, bb[c]));
     }
-    accX[2 * f] += dvr;
-    accX[2 * f + 1] += dvi;
+    if (!act) continue;
+    accX[2 * j] += dvr;
+    accX[2 * j + 1] += dvi;
     if (P.ps_dX) {
       double2* o = reinterpret_cast<double2*>(P.ps_dX) + (size_t)f * P.n + s;
       *o = make_double2(dvr, dvi);
     }
     if (FWD) {
-      accV[4 * f] += vr;
-      accV[4 * f + 1] += vi;
-      accV[4 * f + 2] = fma(vr, vr, accV[4 * f + 2]);
-      accV[4 * f + 3] = fma(vi, vi, accV[4 * f + 3]);
+      accV[4 * j] += vr;
+      accV[4 * j + 1] += vi;
+      accV[4 * j + 2] = fma(vr, vr, accV[4 * j + 2]);
+      accV[4 * j + 3] = fma(vi, vi, accV[4 * j + 3]);
       if (P.ps_v) reinterpret_cast<double2*>(P.ps_v)[(size_t)f * P.n + s] = make_double2(vr, vi);
     }
   }
@@ -189,9 +193,12 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   const int* g2node = reinterpret_cast<const int*>(smem + H.off_g2node);
 
   double accX[2 * kBwFreq], accV[FWD ? 4 * kBwFreq : 1];
-  for (int i = 0; i < 2 * n_f; ++i) accX[i] = 0.0;
-  if (FWD)
-    for (int i = 0; i < 4 * n_f; ++i) accV[i] = 0.0;
+  const int Q = 1 << P.lq, q0 = tid & (Q - 1);
+  for (int j = 0; j * Q < n_f; ++j) {
+    accX[2 * j] = accX[2 * j + 1] = 0.0;
+    if (FWD)
+      for (int k = 0; k < 4; ++k) accV[4 * j + k] = 0.0;
+  }
   double gmu = 0.0, gkx = 0.0, gky = 0.0;
   __shared__ double s_gsum;                  // sum_f Re g_f in frequency order: the R = 1 group's Wb
   __syncthreads();
@@ -213,10 +220,13 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   }
 
   const double beta = P.beta;
-  const long long n_tiles = (P.n + kBlock - 1) / kBlock;
+  const int per_tile = kBlock >> P.lq;
+  const long long n_tiles = (P.n + per_tile - 1) / per_tile;
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const long long s = tile * kBlock + tid;
-    if (s >= P.n) continue;
+    const long long s0 = tile * per_tile + (tid >> P.lq);
+    const bool act = s0 < P.n;
+    if (!act && Q == 1) continue;
+    const long long s = act ? s0 : P.n - 1;      // lanes past the end take part in the shuffles only
     // ------------------------------------------------------------ forward recomputation
     // line energies, and for the lines carrying k_ext the factors G of dE/dK = -G: read from the
     // forward's saved rows, or recomputed from the momenta exactly as the forward forms them
@@ -311,11 +321,15 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
     }
     for (int c = 0; c < H.n_cden; ++c) bb[c] = 0.0;
     if (xr_zero)
-      bwd_phase2<true, FWD>(H, n_f, s, P, Xs, Gs, AXI, AXI2, cden_a, g2, g2cd, pnode, g2node, pW, b, W2, Wb2, bb,
+      bwd_phase2<true, FWD>(H, n_f, s, q0, act, P, Xs, Gs, AXI, AXI2, cden_a, g2, g2cd, pnode, g2node, pW, b, W2, Wb2, bb,
                             accX, accV);
     else
-      bwd_phase2<false, FWD>(H, n_f, s, P, Xs, Gs, AXI, AXI2, cden_a, g2, g2cd, pnode, g2node, pW, b, W2, Wb2, bb,
+      bwd_phase2<false, FWD>(H, n_f, s, q0, act, P, Xs, Gs, AXI, AXI2, cden_a, g2, g2cd, pnode, g2node, pW, b, W2, Wb2, bb,
                              accX, accV);
+    for (int off = 1; off < Q; off <<= 1) {      // the sample's lanes add up their frequencies' parts
+      for (int h = H.g2_const; h < H.n_g2; ++h) Wb2[h] += __shfl_xor_sync(0xffffffffu, Wb2[h], off);
+      for (int c = 0; c < H.n_cden; ++c) bb[c] += __shfl_xor_sync(0xffffffffu, bb[c], off);
+    }
     if (H.g2_const) Wb2[0] = s_gsum;             // R = 1: sum_f Re(conj g_f * 1), as the loop would add it
     // ------------------------------------------------------------ reverse sweep
     double xbar[kBwCombos], fvbar[kBwFv];
@@ -384,6 +398,7 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
       kxb = fma(-eb * ae, Gx[r], kxb);
       kyb = fma(-eb * ae, Gy[r], kyb);
     }
+    if (!act || q0 != 0) continue;
     gmu += mub;
     gkx += kxb;
     gky += kyb;
@@ -396,12 +411,20 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   // -------------------------------------------------------------- block reduction
   const int nval = bwd_nval(n_f, FWD);
   const int warp = tid >> 5, lane = tid & 31;
-  for (int i = 0; i < nval; ++i) {
-    double v = i < 2 * n_f ? accX[i] : (i == 2 * n_f ? gmu : (i == 2 * n_f + 1 ? gkx : gky));
-    if (FWD && i >= 2 * n_f + 3) v = accV[i - 2 * n_f - 3];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) red[warp * nval + i] = v;
+  // lanes of one q0 hold the same frequencies: the warp's sum is theirs
+  auto put = [&](double v, int i, bool mine) {
+    for (int off = 16; off >= Q; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (lane < Q && mine) red[warp * nval + i] = v;
+  };
+  for (int j = 0; j * Q < n_f; ++j) {
+    const int f = j * Q + q0;
+    for (int k = 0; k < 2; ++k) put(accX[2 * j + k], 2 * f + k, f < n_f);
+    if (FWD)
+      for (int k = 0; k < 4; ++k) put(accV[4 * j + k], 2 * n_f + 3 + 4 * f + k, f < n_f);
   }
+  put(gmu, 2 * n_f, q0 == 0);
+  put(gkx, 2 * n_f + 1, q0 == 0);
+  put(gky, 2 * n_f + 2, q0 == 0);
   __syncthreads();
   for (int i = tid; i < nval; i += kBlock) {
     double v = s_late ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;   // late staging: NaN sums
@@ -458,6 +481,19 @@ bool bwd_generic_ok(const tami_diagram* d, int n_f, bool fwd) {
   return true;
 }
 
+// log2 of the lanes that share a sample: each repeats the sample's forward part and reverse sweep and
+// takes every Q-th frequency.  Launches of few samples and many frequencies are one thread's serial
+// walk long; up to 8 lanes, while every lane keeps four frequencies and six blocks per SM hold all
+// threads (order 3, 5000 samples x 200 frequencies 1605 -> 316 us with 8 lanes, 375 with 16; three
+// bubbles, 20 000 x 100, 1133 -> 403 us with 4; five bubbles, 50 000 x 40, 688 -> 524 us with 2; order
+// 4, 20 000 x 16, 399 -> 322 us; but order 5, 10 000 x 4, 303 -> 367 us: a lane with one frequency).
+int bwd_lanes(const tami_diagram* d, int n_f, long long n) {
+  const long long threads = 6LL * kBlock * device_props(d->device).sms;
+  int lq = 0;
+  while (lq < 3 && (8 << lq) <= n_f && n <= (threads >> (lq + 1))) ++lq;
+  return lq;
+}
+
 // Grid of an adjoint launch (the workspace holds its partial rows).  A table the generic kernel
 // cannot take (*generic_ok = false) runs only on the specialised kernel, whose launch is clamped to
 // the workspace's rows: 4 blocks per SM.
@@ -476,7 +512,8 @@ int bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool
   // group the samples alike and the results agree bit for bit
   const int per_sm = fwd ? resident((const void*)bwd_kernel<false, true>)
                          : std::min(resident((const void*)bwd_kernel<false, false>), resident((const void*)bwd_kernel<true, false>));
-  long long tiles = (n + kBlock - 1) / kBlock;
+  const int per_tile = kBlock >> bwd_lanes(d, n_f, n);
+  long long tiles = (n + per_tile - 1) / per_tile;
   long long grid = (long long)dp.sms * per_sm;
   if (grid > tiles) grid = tiles;
   if (grid < 1) grid = 1;
@@ -604,6 +641,7 @@ int tami_backward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed,
     P.saved = saved;
     P.partial = partial;
     P.wait_limit = wait_limit();
+    P.lq = bwd_lanes(d, n_f, n_samples);
     if (saved) bwd_kernel<true, false><<<grid, kBlock, smem, st>>>(P);
     else bwd_kernel<false, false><<<grid, kBlock, smem, st>>>(P);
     e = cudaGetLastError();
@@ -657,6 +695,7 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
     P.ps_dX = per_sample_dX; P.ps_grad = per_sample_grads; P.ps_v = per_sample;
     P.partial = partial;
     P.wait_limit = wait_limit();
+    P.lq = bwd_lanes(d, n_f, n_samples);
     bwd_kernel<false, true><<<grid, kBlock, smem, st>>>(P);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "fused kernel launch");
