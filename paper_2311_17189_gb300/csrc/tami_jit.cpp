@@ -252,12 +252,13 @@ bool ps_first_steps() {
   const char* e = std::getenv("TAMI_JIT_PSFIRST");
   return !(e && !std::strcmp(e, "0"));
 }
-// Spreads a share evenly over a sequence of products: next() says whether the next one is in it.
+// Spreads a share evenly over a sequence of products (to the nearest whole number): next() says
+// whether the next one is in it.
 struct Spread {
-  double share = 1.0, due = 0.0;
+  double share = 1.0, due = 0.5;
   bool next() {
     due += share;
-    if (due < 1.0 - 1e-9) return false;
+    if (due < 1.0) return false;
     due -= 1.0;
     return true;
   }
@@ -302,15 +303,101 @@ double balanced_share(const std::string& code, double other) {
   return std::min(1.0, std::max(0.0, 1.0 - on_fp / products));
 }
 
+// The energy-input kind's value by Horner's rule over the product trie: node v holds S_v = W_v + sum
+// over its children S_child r_child (real at a leaf) and the value is sum_c S_c r_c over the first
+// level, where every group's product R and sum_h W_h R_h take twice the fmas and products at a leaf.
+// A denominator that meets a real S once and nothing else takes S r = (S / |D|^2) conj(D): one
+// product instead of its reciprocal's two.  (The Monte Carlo kinds keep the products R: the adjoint
+// needs them, and the forward's values are the fused pass's bits.) 
+// Two external frequencies, 400 000 rows x 100: 4.79 -> 3.10 ms; order 4, 10^6 rows x 36: 2.67 -> 1.88
+// ms; the evaluation example, 10^6 x 100: 0.818 -> 0.648 ms.
+struct HornerWriter {
+  Out& o;
+  const Table& t;
+  const std::function<std::string(const std::string&, const std::string&)>& MUL;
+  const std::function<std::string(const std::string&)>& NEG;
+  std::vector<std::vector<int>> children;   // of each value: the nodes that continue it
+  std::vector<int> group, uses;             // of each value: its group or -1; of each reciprocal: its factors
+  int names = 0;
+
+  struct Sum { std::string re, im; };       // "": nothing yet (an exact zero)
+
+  HornerWriter(Out& out, const Table& table, const std::function<std::string(const std::string&, const std::string&)>& mul,
+               const std::function<std::string(const std::string&)>& neg)
+      : o(out), t(table), MUL(mul), NEG(neg) {
+    const TableHeader& h = t.h;
+    const int* pnode = t.I(h.off_pnode);
+    const int* g2node = t.I(h.off_g2node);
+    children.resize(h.n_cden + h.n_pnode);
+    group.assign(h.n_cden + h.n_pnode, -1);
+    uses.assign(h.n_cden, 0);
+    for (int k = 0; k < h.n_pnode; ++k) {
+      children[pnode[2 * k]].push_back(h.n_cden + k);
+      ++uses[pnode[2 * k + 1]];
+    }
+    for (int g = h.g2_const; g < h.n_g2; ++g) group[g2node[g]] = g;
+    for (int c = 0; c < h.n_cden; ++c) uses[c] += first_level(c);
+  }
+  bool first_level(int c) const { return group[c] >= 0 || !children[c].empty(); }
+  int factor(int v) const { return v < t.h.n_cden ? v : t.I(t.h.off_pnode)[2 * (v - t.h.n_cden) + 1]; }
+  // whether reciprocal c is only the factor of one leaf
+  bool once(int c) const {
+    if (uses[c] != 1) return false;
+    if (first_level(c)) return children[c].empty();
+    for (int k = 0; k < t.h.n_pnode; ++k)
+      if (factor(t.h.n_cden + k) == c) return children[t.h.n_cden + k].empty();
+    return false;
+  }
+  std::string name(const std::string& value) {
+    const std::string n = "hv" + std::to_string(names++);
+    o("        const double %s = %s;", n.c_str(), value.c_str());
+    return n;
+  }
+  static std::string fma(const std::string& a, const std::string& b, const std::string& c) {
+    return "fma(" + a + ", " + b + ", " + c + ")";
+  }
+  // acc + (child's S) r
+  Sum plus(Sum acc, int v) {
+    const int c = factor(v);
+    const std::string cs = std::to_string(c), rr = "vre" + cs, ri = "vim" + cs;
+    const Sum s = sum(v);
+    if (s.im.empty() && once(c)) {
+      const std::string q = name(MUL(s.re, "r" + cs)), a = "AXI[" + cs + " * n_f + f]";
+      acc.re = name(acc.re.empty() ? MUL(q, "Dr" + cs) : fma(q, "Dr" + cs, acc.re));
+      acc.im = name(acc.im.empty() ? NEG(MUL(q, a)) : fma("-" + q, a, acc.im));
+    } else if (s.im.empty()) {
+      acc.re = name(acc.re.empty() ? MUL(s.re, rr) : fma(s.re, rr, acc.re));
+      acc.im = name(acc.im.empty() ? MUL(s.re, ri) : fma(s.re, ri, acc.im));
+    } else {
+      acc.re = name(fma(s.re, rr, acc.re.empty() ? NEG(MUL(s.im, ri)) : fma("-" + s.im, ri, acc.re)));
+      acc.im = name(fma(s.re, ri, acc.im.empty() ? MUL(s.im, rr) : fma(s.im, rr, acc.im)));
+    }
+    return acc;
+  }
+  Sum sum(int v) {
+    Sum s;
+    if (group[v] >= 0) s.re = "W2_" + std::to_string(group[v]);
+    for (int k : children[v]) s = plus(s, k);
+    return s;
+  }
+  Sum value() {
+    Sum s;
+    if (t.h.g2_const) s.re = "W2_0";
+    for (int c = 0; c < t.h.n_cden; ++c)
+      if (first_level(c)) s = plus(s, c);
+    return s;
+  }
+};
+
 // share: the part of the products, spread evenly over the loop, that is written as imul
 void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
   const TableHeader& h = t.h;
   const bool ia = int_products(h);
   Spread spread{share};
-  auto MUL = [&](const std::string& a, const std::string& b) {
+  const std::function<std::string(const std::string&, const std::string&)> MUL = [&](const std::string& a, const std::string& b) {
     return ia && spread.next() ? "imul(" + a + ", " + b + ")" : a + " * " + b;
   };
-  auto NEG = [&](const std::string& a) {   // sign flip (no arithmetic)
+  const std::function<std::string(const std::string&)> NEG = [&](const std::string& a) {   // sign flip (no arithmetic)
     return "__longlong_as_double(__double_as_longlong(" + a + ") ^ (long long)0x8000000000000000ull)";
   };
   auto S = [](const char* p, int i) { return std::string(p) + std::to_string(i); };
@@ -323,6 +410,7 @@ void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
   const int* g2node = t.I(h.off_g2node);
   const double* cden_a = t.D(h.off_cden_a);
   const int* cden_xk = t.I(h.off_cden_xk);
+  HornerWriter horner(o, t, MUL, NEG);
   o("      for (int f = 0; f < n_f; ++f) {");
   o("        const double Xr = Xs[2 * f]; (void)Xr;");
   if (adj) o("        const double gr = Gs[2 * f], gim = Gs[2 * f + 1], ngr = -gr, ngi = -gim; (void)ngr; (void)ngi;");
@@ -331,8 +419,16 @@ void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
     else if (energy) o("        const double Dr%d = fma(%s, Xs[2 * (%d * n_f + f)], b%d);", c, lit(cden_a[c]).c_str(), cden_xk[c], c);
     else o("        const double Dr%d = fma(%s, Xr, b%d);", c, lit(cden_a[c]).c_str(), c);
     o("        const double r%d = rcp(fma(Dr%d, Dr%d, AXI2[%d * n_f + f]));", c, c, c, c);
+    if (energy && horner.once(c)) continue;
     o("        const double vre%d = %s, vim%d = %s;", c, MUL(S("Dr", c), S("r", c)).c_str(), c,
       NEG(MUL("AXI[" + std::to_string(c) + " * n_f + f]", S("r", c))).c_str());
+  }
+  if (energy) {
+    const HornerWriter::Sum v = horner.value();
+    o("        const double vr = %s, vi = %s;", v.re.empty() ? "0.0" : v.re.c_str(), v.im.empty() ? "0.0" : v.im.c_str());
+    o("        reinterpret_cast<double2*>(ps_v)[(size_t)f * n + s] = make_double2(vr, vi);");
+    o("      }");
+    return;
   }
   for (int k = 0; k < np; ++k) {
     const int src = pnode[2 * k], cc = pnode[2 * k + 1], v = nc + k;
@@ -389,9 +485,7 @@ void emit_phase2(Out& o, const Table& t, int kind, bool xr_zero, double share) {
     o("        if (ps_dX) reinterpret_cast<double2*>(ps_dX)[(size_t)f * n + s] = make_double2(dvr, dvi);");
     o("        }");
   }
-  if (energy) {
-    o("        reinterpret_cast<double2*>(ps_v)[(size_t)f * n + s] = make_double2(vr, vi);");
-  } else if (fwd) {
+  if (fwd) {
     o("        if (act) {");
     o("        accV[4 * f] += vr; accV[4 * f + 1] += vi;");
     o("        accV[4 * f + 2] = fma(vr, vr, accV[4 * f + 2]); accV[4 * f + 3] = fma(vi, vi, accV[4 * f + 3]);");
