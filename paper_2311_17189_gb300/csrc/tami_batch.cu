@@ -69,10 +69,10 @@ struct BatchParams {
 };
 
 // Shared memory: staged table part (table_cap: [0, off_opsb) of the largest table, or [0, off_ops)
-// with streamed programs) | ring [2][ring_chunk] ops | Xs | AXI, AXI2 | CB | W | red
+// with streamed programs) | ring [2][ring_chunk] ops | Xs | AXI, AXI2 | CB | W (red over them)
 size_t batch_smem_bytes(int table_cap, int ring_chunk, int n_f, int max_cden, int max_g2) {
   return (size_t)table_cap + 2 * 8 * (size_t)ring_chunk +
-         sizeof(double) * ((2 + 2 * (size_t)max_cden) * n_f + (size_t)(max_cden + max_g2 + 4) * kBlock);
+         sizeof(double) * ((2 + 2 * (size_t)max_cden) * n_f + (size_t)tile_rows(max_cden, max_g2) * kBlock);
 }
 
 template <bool STREAM>
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kBlock) batch_kernel(const BatchParams P) {
   double* AXI2 = AXI + P.max_cden * n_f;
   double* CB = AXI2 + P.max_cden * n_f;
   double* W = CB + P.max_cden * kBlock;
-  double* red = W + P.max_g2 * kBlock;
+  double* red = CB;                          // between tiles
   for (int i = tid; i < 2 * n_f; i += kBlock) Xs[i] = P.X[i];
   mbar_init(&bar);
   OpRing R;

@@ -55,10 +55,10 @@ struct BwdParams {
 __host__ __device__ __forceinline__ int bwd_nval(int n_f, bool fwd) { return 2 * n_f + 3 + (fwd ? 4 * n_f : 0); }
 
 // Shared memory: table | X, G [n_f][2] | AXI, AXI2 [n_cden][n_f] | red [4 warps][nval].  The table
-// part is [0, off_ops) followed by the adjoint program [off_opsb, bytes) (the forward program is
-// not staged).
+// part is [0, off_p2prog) followed by the adjoint program [off_opsb, bytes) (the forward's programs
+// are not staged).
 __host__ __device__ __forceinline__ size_t bwd_table_smem(const TableHeader& h) {
-  return (size_t)h.off_ops + (size_t)(h.bytes - h.off_opsb);
+  return (size_t)h.off_p2prog + (size_t)(h.bytes - h.off_opsb);
 }
 
 __host__ __device__ __forceinline__ size_t bwd_smem_bytes(const TableHeader& h, int n_f, bool fwd) {
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   let_next_kernel_start();
   __shared__ int s_late;                     // set when the staging wait of this block ran out
   if (tid == 0) s_late = 0;
-  if (!stage_table(smem, P.table, H.off_ops, &s_late, P.wait_limit, P.table + H.off_opsb, H.bytes - H.off_opsb)) {
+  if (!stage_table(smem, P.table, H.off_p2prog, &s_late, P.wait_limit, P.table + H.off_opsb, H.bytes - H.off_opsb)) {
     nan_row(P.partial + (size_t)blockIdx.x * bwd_nval(n_f, FWD), bwd_nval(n_f, FWD));
     return;
   }
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kBlock, TAMI_BWD_MIN_BLOCKS) bwd_kernel(const 
   const double* cden_a = reinterpret_cast<const double*>(smem + H.off_cden_a);
   const int* g1 = reinterpret_cast<const int*>(smem + H.off_g1);
   const int* g1_tgt = reinterpret_cast<const int*>(smem + H.off_g1_tgt);
-  const int2* opsb = reinterpret_cast<const int2*>(smem + H.off_ops);   // staged right after [0, off_ops)
+  const int2* opsb = reinterpret_cast<const int2*>(smem + H.off_p2prog);   // staged right after [0, off_p2prog)
   const int* g1_node = reinterpret_cast<const int*>(smem + H.off_g1_node);
   const double* leafA = reinterpret_cast<const double*>(smem + H.off_leafA);
   const int* g1rd = reinterpret_cast<const int*>(smem + H.off_g1rd);

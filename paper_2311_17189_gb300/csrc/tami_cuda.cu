@@ -56,11 +56,11 @@ __host__ __device__ __forceinline__ size_t fwd_table_smem(const TableHeader& h, 
   return ring_chunk ? (size_t)h.off_ops + 2 * 8 * (size_t)ring_chunk : (size_t)h.off_opsb;
 }
 
-// Shared memory: table | Xs [n_xk][n_f][2] | AXI, AXI2 [n_cden][n_f] | CB [n_cden][S] | W [n_g2][S] |
-// red [4][S]
+// Shared memory: table | Xs [n_xk][n_f][2] | AXI, AXI2 [n_cden][n_f] | CB [n_cden][S] | W [n_g2][S],
+// and over CB and W, after the last tile, red [4][S]
 __host__ __device__ __forceinline__ size_t fwd_smem_bytes(const TableHeader& h, int n_f, int ring_chunk) {
   return fwd_table_smem(h, ring_chunk) +
-         sizeof(double) * ((2 * (size_t)h.n_xk + 2 * (size_t)h.n_cden) * n_f + (size_t)(h.n_cden + h.n_g2 + 4) * kBlock);
+         sizeof(double) * ((2 * (size_t)h.n_xk + 2 * (size_t)h.n_cden) * n_f + (size_t)tile_rows(h.n_cden, h.n_g2) * kBlock);
 }
 
 // A block whose staging failed or came late leaves NaN partial sums, and with them NaN means: no
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
   double* AXI2 = AXI + H.n_cden * P.n_f;
   double* CB = AXI2 + H.n_cden * P.n_f;
   double* W = CB + H.n_cden * kBlock;
-  double* red = W + H.n_g2 * kBlock;
+  double* red = CB;                          // after the last tile
   const TableView T = table_view(smem, H);
   stage_freqs(H, T, P.X, P.n_f, Xs);
   const FreqMap M = freq_map(P.n_f, tid);

@@ -35,6 +35,7 @@ struct TableView {
   const int* g2cd;
   const int* pnode;
   const int* g2node;
+  const int* p2prog;
 };
 
 __device__ __forceinline__ TableView table_view(const unsigned char* t, const TableHeader& H) {
@@ -62,6 +63,7 @@ __device__ __forceinline__ TableView table_view(const unsigned char* t, const Ta
   v.g2cd = reinterpret_cast<const int*>(t + H.off_g2cd);
   v.pnode = reinterpret_cast<const int*>(t + H.off_pnode);
   v.g2node = reinterpret_cast<const int*>(t + H.off_g2node);
+  v.p2prog = reinterpret_cast<const int*>(t + H.off_p2prog);
   return v;
 }
 
@@ -196,6 +198,13 @@ __device__ __forceinline__ FreqMap freq_map(int n_f, int tid) {
   return m;
 }
 
+// Rows of kBlock doubles behind the frequency constants: CB and W, and over them, when no tile is in
+// flight, the 4 rows of block_reduce_store (shared memory a block does not take is L1 for the tile's
+// per-thread arrays).
+__host__ __device__ __forceinline__ int tile_rows(int n_cden, int n_g2) {
+  return n_cden + n_g2 > 4 ? n_cden + n_g2 : 4;
+}
+
 struct TileArgs {
   double t, tp, mu, kx, ky, beta;
   unsigned long long seed, offset;  // sample s of the tile stream is Philox counter offset + s
@@ -254,33 +263,46 @@ __device__ __forceinline__ bool freq_constants(const TableHeader& H, const Table
 // first (g2_const).  The products run on the integer pipes (imul, the FP64 unit's bits), beside the
 // sums' fmas (two external frequencies, 250 000 rows x 100: 4.25 -> 3.37 ms; order-4 forward, 10^6
 // samples x 21 frequencies: 2.82 -> 2.50 ms).
-// S: the samples of a tile (the stride of CB and W).
-template <bool XR_ZERO, int S>
-__device__ __forceinline__ void phase2_sample(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
-                                              int f, const double* Xs, const double* AXI, const double* AXI2,
-                                              const double* CB, const double* W, double& vr_out, double& vi_out) {
-  // values: [0, n_cden) the reciprocals 1/D_c, then the product nodes
-  double vre[kMaxCplxDens + kMaxProdNodes], vim[kMaxCplxDens + kMaxProdNodes];
+//
+// The walk follows phase2_program: each group's weight is added as soon as its product is there, the
+// running product stays in registers, and of the products only those that a later group starts from
+// are kept (order 4: 1 of 7).  With every product in per-thread memory beside the reciprocals the
+// resident threads' arrays were larger than L1 -- half of the loads went to L2, 13.4 GB in 2.5 ms --
+// and with the loops unrolled and two samples a step the warps waited on instruction fetch as often
+// as on the FP64 unit (2.4 stalls per issue); now 0.2, and 84 % of the loads hit.  Order-4 forward,
+// 10^6 samples x 21 frequencies: 2.51 -> 2.28 ms; order 2, 10^6 x 3: 232 -> 211 us; 28 streams of
+// 16384 samples x 32 frequencies: 5.45 -> 5.07 ms.
+template <bool XR_ZERO>
+__device__ __forceinline__ void phase2_walk(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
+                                            int f, const double* Xs, const double* AXI, const double* AXI2,
+                                            const double* CB, const double* W, double& vr_out, double& vi_out) {
+  // values: [0, n_cden) the reciprocals 1/D_c, then the products that later groups start from
+  double2 val[kMaxCplxDens + kMaxProdNodes];
+#pragma unroll 1
   for (int c = 0; c < H.n_cden; ++c) {
-    const double b = CB[c * S + sl];
+    const double b = CB[c * kBlock + sl];
     // D = g_c Y_{k_c f} + b
     const double Dr = XR_ZERO ? b : fma(T.cden_a[c], Xs[2 * (T.cden_xk[c] * A.n_f + f)], b);
     const double r = rcp(fma(Dr, Dr, AXI2[c * A.n_f + f]));
-    vre[c] = imul(Dr, r);
-    vim[c] = neg_bits(imul(AXI[c * A.n_f + f], r));
-  }
-  for (int k = 0; k < H.n_pnode; ++k) {
-    const int src = T.pnode[2 * k], c = T.pnode[2 * k + 1];
-    const double ar = vre[src], ai = vim[src], br = vre[c], bi = vim[c];
-    vre[H.n_cden + k] = fma(ar, br, neg_bits(imul(ai, bi)));
-    vim[H.n_cden + k] = fma(ar, bi, imul(ai, br));
+    val[c] = make_double2(imul(Dr, r), neg_bits(imul(AXI[c * A.n_f + f], r)));
   }
   double vr = H.g2_const ? W[sl] : 0.0, vi = 0.0;
+  double2 run = make_double2(0.0, 0.0);
+  const int* p = T.p2prog;
+#pragma unroll 1
   for (int hg = H.g2_const; hg < H.n_g2; ++hg) {
-    const double w = W[hg * S + sl];
-    const int v = T.g2node[hg];
-    vr = fma(w, vre[v], vr);
-    vi = fma(w, vim[v], vi);
+    const double w = W[hg * kBlock + sl];
+    const int e = *p++;
+    if ((e & 0xffff) != kP2Last) run = val[e & 0xffff];
+#pragma unroll 1
+    for (int k = e >> 16; k > 0; --k) {
+      const int x = *p++, slot = x >> 8;
+      const double2 q = val[x & 255];
+      run = make_double2(fma(run.x, q.x, neg_bits(imul(run.y, q.y))), fma(run.x, q.y, imul(run.y, q.x)));
+      if (slot) val[slot] = run;
+    }
+    vr = fma(w, run.x, vr);
+    vi = fma(w, run.y, vi);
   }
   vr_out = vr;
   vi_out = vi;
@@ -411,8 +433,6 @@ __device__ __forceinline__ void fwd_tile(const TableHeader& H, const TableView& 
   __syncthreads();
 }
 
-// Two samples per iteration give the FP64 pipe two independent dependency chains; the sums are
-// still taken sample by sample, in the same order.
 // Swap the running sums of the thread's two frequencies (selects, no FP64 work).
 __device__ __forceinline__ void swap_sums(bool sw, double* a, double* b) {
   for (int k = 0; k < 4; ++k) {
@@ -435,29 +455,15 @@ __device__ __forceinline__ void phase2_loop(const TableHeader& H, const TableVie
     double cur[4], oth[4];
     for (int k = 0; k < 4; ++k) { cur[k] = acc[0][k]; oth[k] = acc[1][k]; }
     bool crossed = false;
-    int j = 0;
-    for (; j + 1 < A.n_f; j += 2) {
-      const int pa = M.p0 + j, pb = pa + 1;
-      const int fa = pa / kBlock, sla = pa % kBlock, fb = pb / kBlock, slb = pb % kBlock;
-      double ar, ai, br, bi;
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, slb, fb, Xs, AXI, AXI2, CB, W, br, bi);
-      const bool sa = sla == 0 && j > 0, sb = slb == 0;
-      swap_sums(sa, cur, oth);
-      crossed |= sa;
-      if (s0 + sla < A.n) phase2_store(A, fa, s0 + sla, ar, ai, cur);
-      swap_sums(sb, cur, oth);
-      crossed |= sb;
-      if (s0 + slb < A.n) phase2_store(A, fb, s0 + slb, br, bi, cur);
-    }
-    if (j < A.n_f) {
-      const int pa = M.p0 + j, fa = pa / kBlock, sla = pa % kBlock;
-      double ar, ai;
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, sla, fa, Xs, AXI, AXI2, CB, W, ar, ai);
-      const bool sa = sla == 0 && j > 0;
-      swap_sums(sa, cur, oth);
-      crossed |= sa;
-      if (s0 + sla < A.n) phase2_store(A, fa, s0 + sla, ar, ai, cur);
+#pragma unroll 1
+    for (int j = 0; j < A.n_f; ++j) {
+      const int p = M.p0 + j, f = p / kBlock, sl = p % kBlock;
+      double vr, vi;
+      phase2_walk<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, vr, vi);
+      const bool sw = sl == 0 && j > 0;
+      swap_sums(sw, cur, oth);
+      crossed |= sw;
+      if (s0 + sl < A.n) phase2_store(A, f, s0 + sl, vr, vi, cur);
     }
     swap_sums(crossed, cur, oth);     // back to acc[0] = frequency f0, acc[1] = f0 + 1
     for (int k = 0; k < 4; ++k) { acc[0][k] = cur[k]; acc[1][k] = oth[k]; }
@@ -467,17 +473,11 @@ __device__ __forceinline__ void phase2_loop(const TableHeader& H, const TableVie
     const int f = M.f0 + fi * M.fstep;
     int sl = fi ? M.sb1 : M.sb0;
     const int se = fi ? M.se1 : M.se0;
-    for (; sl + M.sstep < se && s0 + sl + M.sstep < A.n; sl += 2 * M.sstep) {
-      double ar, ai, br, bi;
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl + M.sstep, f, Xs, AXI, AXI2, CB, W, br, bi);
-      phase2_store(A, f, s0 + sl, ar, ai, acc[fi]);
-      phase2_store(A, f, s0 + sl + M.sstep, br, bi, acc[fi]);
-    }
+#pragma unroll 1
     for (; sl < se && s0 + sl < A.n; sl += M.sstep) {
-      double ar, ai;
-      phase2_sample<XR_ZERO, kBlock>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, ar, ai);
-      phase2_store(A, f, s0 + sl, ar, ai, acc[fi]);
+      double vr, vi;
+      phase2_walk<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, CB, W, vr, vi);
+      phase2_store(A, f, s0 + sl, vr, vi, acc[fi]);
     }
   }
 }
@@ -495,6 +495,40 @@ constexpr int kCoopFreqPerThread = kCoopMaxFreq / kCoopWarps;
 
 template <bool V>
 struct BoolConst { static constexpr bool value = V; };
+
+// Phase 2 of the small tile: phase2_walk's values and sums, bit for bit, node by node.  A block's
+// four warps wait on latency, not on L1: unrolled loops over all nodes, then over all groups, take
+// 3.02 ms with two external frequencies (250 000 rows x 100), the walk 3.12 ms.
+template <bool XR_ZERO>
+__device__ __forceinline__ void phase2_nodes(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
+                                             int f, const double* Xs, const double* AXI, const double* AXI2,
+                                             const double* CB, const double* W, double& vr_out, double& vi_out) {
+  // values: [0, n_cden) the reciprocals 1/D_c, then the product nodes
+  double vre[kMaxCplxDens + kMaxProdNodes], vim[kMaxCplxDens + kMaxProdNodes];
+  for (int c = 0; c < H.n_cden; ++c) {
+    const double b = CB[c * kCoopSamples + sl];
+    // D = g_c Y_{k_c f} + b
+    const double Dr = XR_ZERO ? b : fma(T.cden_a[c], Xs[2 * (T.cden_xk[c] * A.n_f + f)], b);
+    const double r = rcp(fma(Dr, Dr, AXI2[c * A.n_f + f]));
+    vre[c] = imul(Dr, r);
+    vim[c] = neg_bits(imul(AXI[c * A.n_f + f], r));
+  }
+  for (int k = 0; k < H.n_pnode; ++k) {
+    const int src = T.pnode[2 * k], c = T.pnode[2 * k + 1];
+    const double ar = vre[src], ai = vim[src], br = vre[c], bi = vim[c];
+    vre[H.n_cden + k] = fma(ar, br, neg_bits(imul(ai, bi)));
+    vim[H.n_cden + k] = fma(ar, bi, imul(ai, br));
+  }
+  double vr = H.g2_const ? W[sl] : 0.0, vi = 0.0;
+  for (int hg = H.g2_const; hg < H.n_g2; ++hg) {
+    const double w = W[hg * kCoopSamples + sl];
+    const int v = T.g2node[hg];
+    vr = fma(w, vre[v], vr);
+    vi = fma(w, vim[v], vi);
+  }
+  vr_out = vr;
+  vi_out = vi;
+}
 
 struct CoopBuffers {   // each [count][kCoopSamples]
   double *K, *E, *x, *fv, *rr, *W1, *W, *CB;
@@ -612,7 +646,7 @@ __device__ __forceinline__ void coop_tile(const TableHeader& H, const TableView&
     constexpr bool XR_ZERO = decltype(zero)::value;
     for (int f = w, i = 0; f < A.n_f; f += kCoopWarps, ++i) {
       double vr, vi;
-      phase2_sample<XR_ZERO, S>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, vr, vi);
+      phase2_nodes<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, vr, vi);
       if (!active) continue;
       if (ENERGY_IN) {
         double2* o = reinterpret_cast<double2*>(A.per_sample) + (size_t)f * A.n + s;

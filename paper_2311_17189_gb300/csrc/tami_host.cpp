@@ -631,6 +631,11 @@ int flatten(tami_diagram* d) {
   h.n_g1rd = ng1rd;
   h.n_g2 = (int)g2s.size(); h.n_g2cd = ng2cd;
   h.n_pnode = (int)pnodes.size();
+  std::vector<int> pnode_words;
+  for (auto& pn : pnodes) { pnode_words.push_back(pn.first); pnode_words.push_back(pn.second); }
+  const std::vector<int> p2prog = phase2_program(n_cd, g2_const, (int)g2s.size(), g2node.data(), pnode_words.data(),
+                                                 h.n_pnode, &h.n_p2live);
+  h.n_p2prog = (int)p2prog.size();
   h.g2_const = g2_const;
   h.max_der = max_der;
   Blob B;
@@ -663,7 +668,8 @@ int flatten(tami_diagram* d) {
   h.off_g2cd_p = B.reserve(sizeof(double) * ng2cd);
   h.off_pnode = B.reserve(sizeof(int) * 2 * h.n_pnode);
   h.off_g2node = B.reserve(sizeof(int) * h.n_g2);
-  // the two pole-DAG programs last: a forward kernel stages [0, off_opsb), an adjoint [0, off_ops)
+  h.off_p2prog = B.reserve(sizeof(int) * h.n_p2prog);
+  // the two pole-DAG programs last: a forward kernel stages [0, off_opsb), an adjoint [0, off_p2prog)
   // and [off_opsb, bytes), and a program too large for shared memory is streamed from off_ops
   h.off_ops = B.reserve(sizeof(int) * 2 * h.n_ops);
   h.off_opsb = B.reserve(sizeof(int) * 2 * h.n_ops);
@@ -757,11 +763,9 @@ int flatten(tami_diagram* d) {
     }
     B.at<int>(h.off_g2)[h.n_g2] = pos;
   }
-  for (int k = 0; k < h.n_pnode; ++k) {
-    B.at<int>(h.off_pnode)[2 * k] = pnodes[k].first;
-    B.at<int>(h.off_pnode)[2 * k + 1] = pnodes[k].second;
-  }
+  for (int k = 0; k < 2 * h.n_pnode; ++k) B.at<int>(h.off_pnode)[k] = pnode_words[k];
   for (int g = 0; g < h.n_g2; ++g) B.at<int>(h.off_g2node)[g] = g2node[g];
+  for (int k = 0; k < h.n_p2prog; ++k) B.at<int>(h.off_p2prog)[k] = p2prog[k];
   d->blob.swap(B.b);
   {
     std::string why;

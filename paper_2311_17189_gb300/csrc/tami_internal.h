@@ -72,8 +72,8 @@ struct SymTerm {
 // Flattened table.  All offsets are byte offsets into one blob, 16-byte aligned, so the blob
 // can be moved into shared memory with bulk copies.  Integer records are int32.  The two
 // pole-DAG programs are the last sections, [off_ops, off_opsb) and [off_opsb, bytes), everything
-// else lies in [0, off_ops): a forward kernel stages [0, off_opsb), an adjoint kernel [0, off_ops)
-// and [off_opsb, bytes), and a forward whose program does not fit beside its tiles stages
+// else lies in [0, off_ops), the forward's phase-2 program at its end: a forward kernel stages
+// [0, off_opsb), an adjoint kernel [0, off_p2prog) and [off_opsb, bytes), and a forward whose program does not fit beside its tiles stages
 // [0, off_ops) and streams the program in chunks.
 struct TableHeader {
   int N, nv, m;
@@ -88,6 +88,7 @@ struct TableHeader {
   int n_slots, n_nodes;        // forward value slots (most live in one group); DAG nodes over all groups
   int n_g2, n_g2cd;
   int n_pnode;      // phase-2 product nodes
+  int n_p2prog, n_p2live;   // words of the forward's phase-2 program, product slots it needs
   int g2_const;     // 1 if group 0 of phase 2 has no frequency-dependent factor (R = 1)
   int max_der;
   int n_ext;        // external frequencies per frequency row (the last n_ext variables)
@@ -120,9 +121,52 @@ struct TableHeader {
   int off_g2cd_p;     // double [n_g2cd]          the same powers as doubles
   int off_pnode;      // int32 [n_pnode][2]      product node k: value[n_cden+k] = value[src] * value[c]
   int off_g2node;     // int32 [n_g2]             value index of each group's product (-1: R = 1)
+  int off_p2prog;     // int32 [n_p2prog]         the forward's phase-2 program (phase2_program)
   int off_ops;        // int2 [n_ops]            pole-tree program, forward encoding (kOp*)
   int off_opsb;       // int2 [n_ops]            the same program, adjoint encoding (kOpb*)
 };
+
+// The forward kernels' walk over the product trie: per frequency-dependent group a word
+// source | factors << 16, then a word c | slot << 8 per factor.  The running product starts as
+// value[source] (kP2Last: it goes on from the previous group's) and takes the factors 1/D_c in turn;
+// a product that a later group starts from is also written to value[slot], n_cden <= slot < n_cden +
+// *n_live (slot 0: not written).  Values below n_cden are the reciprocals.
+constexpr int kP2Last = 0xffff;
+inline std::vector<int> phase2_program(int n_cden, int g2_const, int n_g2, const int* g2node, const int* pnode,
+                                       int n_pnode, int* n_live) {
+  struct Step { int source; bool last; std::vector<int> nodes; };
+  std::vector<Step> steps;
+  std::vector<char> have(n_cden + n_pnode, 0);
+  std::vector<int> last_read(n_cden + n_pnode, -1), slot(n_cden + n_pnode, 0);
+  for (int c = 0; c < n_cden; ++c) have[c] = 1;
+  for (int g = g2_const, run = -1; g < n_g2; ++g) {
+    Step s;
+    int v = g2node[g];
+    for (; !have[v]; v = pnode[2 * (v - n_cden)]) { s.nodes.insert(s.nodes.begin(), v); have[v] = 1; }
+    s.source = v;
+    s.last = v == run;
+    if (!s.last) last_read[v] = (int)steps.size();
+    run = g2node[g];
+    steps.push_back(s);
+  }
+  std::vector<int> prog, free_slots;
+  *n_live = 0;
+  for (int i = 0; i < (int)steps.size(); ++i) {
+    const Step& s = steps[i];
+    const bool product = s.source >= n_cden;
+    prog.push_back((s.last ? kP2Last : product ? slot[s.source] : s.source) | (int)s.nodes.size() << 16);
+    if (!s.last && product && last_read[s.source] == i) free_slots.push_back(slot[s.source]);
+    for (int v : s.nodes) {
+      if (last_read[v] >= 0) {
+        if (free_slots.empty()) free_slots.push_back(n_cden + (*n_live)++);
+        slot[v] = free_slots.back();
+        free_slots.pop_back();
+      }
+      prog.push_back(pnode[2 * (v - n_cden) + 1] | slot[v] << 8);
+    }
+  }
+  return prog;
+}
 
 }  // namespace tami
 

@@ -39,15 +39,19 @@ bool in(long long v, long long lo, long long hi) { return v >= lo && v < hi; }
 
 bool validate_table(const TableHeader& h, const unsigned char* blob, size_t size, std::string* why) {
   // every section but the two programs lies in [0, off_ops); the programs are [off_ops, off_opsb)
-  // and [off_opsb, bytes) (the kernels stage these ranges by themselves)
-  const size_t prog = (size_t)h.off_ops;
-  Reader R{blob, prog <= size ? prog : 0};
+  // and [off_opsb, bytes), and the forward's phase-2 program ends at off_ops (the kernels stage
+  // these ranges by themselves)
+  const size_t prog = (size_t)h.off_ops, p2 = (size_t)h.off_p2prog;
+  Reader R{blob, p2 <= prog && prog <= size ? p2 : 0};
   auto bad = [&](const std::string& w) { R.fail(w); };
   if ((size_t)h.bytes != size) bad("header size differs from the blob");
   const size_t prog_bytes = (8 * (size_t)std::max(h.n_ops, 0) + 15) & ~size_t(15);
   if (h.off_ops < 0 || (h.off_ops & 15) != 0 || (size_t)h.off_opsb != prog + prog_bytes ||
       (size_t)h.bytes != prog + 2 * prog_bytes + 16)
     bad("pole-DAG programs are not the last sections");
+  if (h.off_p2prog < 0 || (h.off_p2prog & 15) != 0 || h.n_p2prog < 0 ||
+      p2 + ((4 * (size_t)h.n_p2prog + 15) & ~size_t(15)) != prog)
+    bad("phase-2 program not before the pole-DAG programs");
   if (!in(h.N, 1, kMaxLines + 1) || !in(h.nv, 2, kMaxVars + 1) || !in(h.n_ext, 1, kMaxExt + 1) ||
       h.m != h.nv - h.n_ext || h.m < 1)
     bad("line or variable count");
@@ -82,6 +86,7 @@ bool validate_table(const TableHeader& h, const unsigned char* blob, size_t size
   const int* g2cd = R.at<int>(h.off_g2cd, 2 * (size_t)h.n_g2cd, "g2cd");
   const int* pnode = R.at<int>(h.off_pnode, 2 * (size_t)h.n_pnode, "pnode");
   const int* g2node = R.at<int>(h.off_g2node, h.n_g2, "g2node");
+  const int* p2prog = RP.at<int>(h.off_p2prog, h.n_p2prog, "p2prog");
   if (!R.ok) { *why = R.why; return false; }
 
   std::vector<char> computed(h.N, 0);
@@ -171,6 +176,12 @@ bool validate_table(const TableHeader& h, const unsigned char* blob, size_t size
     if (empty ? g2node[hg] != -1 : !in(g2node[hg], 0, h.n_cden + h.n_pnode)) bad("group product node");
     for (int q = g2[hg]; q < g2[hg + 1]; ++q)
       if (!in(g2cd[2 * q], 0, h.n_cden) || g2cd[2 * q + 1] < 1) bad("complex denominator power");
+  }
+  if (R.ok) {
+    int live = 0;
+    const std::vector<int> ref = phase2_program(h.n_cden, h.g2_const, h.n_g2, g2node, pnode, h.n_pnode, &live);
+    if (live != h.n_p2live || (int)ref.size() != h.n_p2prog || !std::equal(ref.begin(), ref.end(), p2prog))
+      bad("phase-2 program");
   }
   if (!R.ok) *why = R.why;
   return R.ok;
