@@ -207,6 +207,7 @@ struct tami_batch {
   int chunk = 0, grid = 0, n_items = 0;
   int table_cap = 0, max_cden = 0, max_g2 = 0;   // over the diagrams the persistent kernel runs
   int ring_chunk = 0;                              // streamed programs: ops per ring buffer
+  int p2_bytes = 0;                                // of table_cap: the phase-2 programs, not counted by the limits
   std::vector<int> spec;                           // 1: the diagram runs its specialised kernel
   std::vector<tami::JitHandle> jit;                // those kernels, kept loaded by the batch
   std::vector<int> jit_grid;
@@ -326,7 +327,7 @@ int build(tami_batch* b, int chunk, int grid_cap, bool with_spec) {
   // grid: resident blocks, capped
   DeviceProps dp = device_props(b->device);
   b->smem = batch_smem_bytes(b->table_cap, b->ring_chunk, n_f, b->max_cden, b->max_g2);
-  if (b->smem > dp.smem_optin) {
+  if (counted_smem(b->smem, b->max_cden, b->max_g2, b->p2_bytes) > dp.smem_optin) {
     set_error("largest table and tiles exceed shared memory even with the pole-DAG programs streamed");
     return TAMI_EUNSUPPORTED;
   }
@@ -549,23 +550,33 @@ int tami_batch_plan(const tami_diagram* const* ds, int n_d, const int64_t* sampl
   }
   // staging: every forward program resident beside the tiles when the largest fits (and streaming
   // is not forced), else the programs streamed through the ring
-  int cap_res = 0, cap_prog = 0;
+  int cap_res = 0, cap_prog = 0, less_res = 0, less_prog = 0;   // less: without the phase-2 programs
   for (int d = 0; d < n_d; ++d) {
     if (b->spec[d]) continue;
     cap_res = std::max(cap_res, ds[d]->hdr.off_opsb);
     cap_prog = std::max(cap_prog, ds[d]->hdr.off_ops);
+    less_res = std::max(less_res, ds[d]->hdr.off_opsb - (ds[d]->hdr.off_ops - ds[d]->hdr.off_p2prog));
+    less_prog = std::max(less_prog, ds[d]->hdr.off_p2prog);
     b->max_cden = std::max(b->max_cden, ds[d]->hdr.n_cden);
     b->max_g2 = std::max(b->max_g2, ds[d]->hdr.n_g2);
   }
   {
     const size_t optin = device_props(b->device).smem_optin;
+    const int p2_res = cap_res - less_res, p2_prog = cap_prog - less_prog;
+    auto count = [&](int cap, int chunk, int less) {
+      return counted_smem(batch_smem_bytes(cap, chunk, n_f, b->max_cden, b->max_g2), b->max_cden, b->max_g2, (size_t)less);
+    };
+    // a program smaller than the ring may fit resident only
     if (staging_mode() != TAMI_STAGING_STREAMED &&
-        batch_smem_bytes(cap_res, 0, n_f, b->max_cden, b->max_g2) <= optin) {
+        (count(cap_res, 0, 0) <= optin ||
+         (count(cap_res, 0, p2_res) <= optin && count(cap_prog, ring_chunk_ops(), p2_prog) > optin))) {
       b->table_cap = cap_res;
       b->ring_chunk = 0;
+      b->p2_bytes = p2_res;
     } else {
       b->table_cap = cap_prog;
       b->ring_chunk = ring_chunk_ops();
+      b->p2_bytes = p2_prog;
     }
   }
   e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);

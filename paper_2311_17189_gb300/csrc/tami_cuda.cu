@@ -297,20 +297,23 @@ __global__ void sample_energies_kernel(const FwdParams P, double* E) {
 // ------------------------------------------------------------------------------- host glue
 // How the generic forward stages a table: the program resident beside the tiles when it fits
 // (and streaming is not forced), else streamed through the ring; ring_chunk = 0 means resident.
-// Returns false when even the streamed layout exceeds shared memory.
-bool fwd_staging(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem) {
+// Returns false when even the streamed layout exceeds shared memory.  counted: the shared memory that
+// the limits count (counted_smem).
+bool fwd_staging(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem, size_t* counted = nullptr) {
   const size_t optin = device_props(d->device).smem_optin;
-  const int mode = staging_mode();
-  if (mode != TAMI_STAGING_STREAMED && fwd_smem_bytes(d->hdr, n_f, 0) <= optin) {
-    *ring_chunk = 0;
-    *smem = fwd_smem_bytes(d->hdr, n_f, 0);
-    return true;
-  }
-  *ring_chunk = ring_chunk_ops();
-  *smem = fwd_smem_bytes(d->hdr, n_f, *ring_chunk);
-  if (*smem > optin) {
+  const TableHeader& h = d->hdr;
+  const size_t p2 = (size_t)(h.off_ops - h.off_p2prog);
+  auto count = [&](int chunk, size_t less) { return counted_smem(fwd_smem_bytes(h, n_f, chunk), h.n_cden, h.n_g2, less); };
+  // a program smaller than the ring may fit resident only
+  const bool resident = staging_mode() != TAMI_STAGING_STREAMED &&
+                        (count(0, 0) <= optin || (count(0, p2) <= optin && count(ring_chunk_ops(), p2) > optin));
+  *ring_chunk = resident ? 0 : ring_chunk_ops();
+  *smem = fwd_smem_bytes(h, n_f, *ring_chunk);
+  const size_t limit = count(*ring_chunk, p2);
+  if (counted) *counted = limit;
+  if (limit > optin) {
     set_error("term table and tiles exceed shared memory even with the pole-DAG program streamed: " +
-              std::to_string(*smem) + " bytes (at most " + std::to_string(optin) + ")");
+              std::to_string(limit) + " bytes (at most " + std::to_string(optin) + ")");
     return false;
   }
   return true;
@@ -381,9 +384,10 @@ int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max
 // run it, whose launch is clamped to the rows of the workspace: 4 blocks per SM.
 int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nullptr, bool coop = true) {
   DeviceProps dp = device_props(d->device);
-  size_t smem = 0;
+  size_t smem = 0, counted = 0;
   int chunk = 0;
-  const bool ok = fwd_staging(d, n_f, &chunk, &smem);
+  const bool ok = fwd_staging(d, n_f, &chunk, &smem, &counted);
+  if (!coop) smem = counted;   // the fixed array's limit
   if (generic_ok) *generic_ok = ok;
   if (!ok) {
     const long long tiles = (n + kBlock - 1) / kBlock;

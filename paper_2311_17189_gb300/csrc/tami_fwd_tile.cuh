@@ -204,6 +204,12 @@ __device__ __forceinline__ FreqMap freq_map(int n_f, int tid) {
 __host__ __device__ __forceinline__ int tile_rows(int n_cden, int n_g2) {
   return n_cden + n_g2 > 4 ? n_cden + n_g2 : 4;
 }
+// What the size limits of the entry points count for a block: the four rows beside the tile's, and no
+// phase-2 program.  Never less than the block takes (a row is 1 KB, the program's words are fewer
+// than 4 for every row), and the limits do not depend on how a kernel lays out its scratch.
+inline size_t counted_smem(size_t taken, int n_cden, int n_g2, size_t p2_bytes) {
+  return taken + sizeof(double) * kBlock * (size_t)(n_cden + n_g2 + 4 - tile_rows(n_cden, n_g2)) - p2_bytes;
+}
 
 struct TileArgs {
   double t, tp, mu, kx, ky, beta;
