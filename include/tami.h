@@ -398,14 +398,14 @@ int tami_set_table_staging(int mode, int chunk_ops);
 
 /* Test hook (not a term of the paper): bound the first stage of every mbarrier wait of the generic
  * kernels' table staging to `first_stage_spins` polls (0 .. 2^24; -1 restores the default 2^24).
- * A wait that runs out sets the call's status word (TAMI_ETIMEOUT in the device status; the
- * reduced outputs of that launch become NaN) and then waits again, bounded by 2^24 polls, for the
+ * A wait that runs out is noted by its block, whose partial sums become NaN and with them the
+ * reduced outputs of that launch (a batch plan sets its status word to TAMI_ETIMEOUT), and then waits again, bounded by 2^24 polls, for the
  * copy to land, so a completed copy is still used safely.  With 0 every staging wait "runs out"
  * on a valid copy, which lets a test drive that path without any fault.  Plans (tami_batch_plan)
  * take the value at planning time; the other calls at each launch.  Process-wide. */
 int tami_debug_set_wait_limit(int64_t first_stage_spins);
 
-/* Diagnostic: the kernels' exponential for t <= 0 (table-driven after Tang, ACM TOMS 1989), applied
+/* Diagnostic: the kernels' exponential for t <= 0 (table-driven, in 64-bit fixed point), applied
  * elementwise: y = e^t, em = e^t - 1, and y_plain = e^t from the variant that does not form
  * e^t - 1 (the kernels use it where only e^t is needed; it must equal y bit for bit).
  * t, y, em, y_plain: device double [n]; y_plain may be NULL.  Used by the tests to check them
