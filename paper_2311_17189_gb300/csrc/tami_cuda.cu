@@ -121,12 +121,12 @@ __global__ void __launch_bounds__(kBlock) fwd_kernel(const FwdParams P) {
 }
 
 // Shared memory of coop_kernel: table | Xs | AXI, AXI2 | the tile's buffers
-__host__ __device__ __forceinline__ size_t coop_smem_bytes(const TableHeader& h, int n_f, int ring_chunk) {
+__host__ __device__ __forceinline__ size_t coop_smem_bytes(const TableHeader& h, int n_f, int ring_chunk, bool walk) {
   return fwd_table_smem(h, ring_chunk) + sizeof(double) * ((2 * (size_t)h.n_xk + 2 * (size_t)h.n_cden) * n_f +
-                                                (size_t)coop_rows(h) * kCoopSamples);
+                                                (size_t)coop_rows(h, walk) * kCoopSamples);
 }
 
-template <bool ENERGY_IN, bool SAVE, bool STREAM>
+template <bool ENERGY_IN, bool SAVE, bool STREAM, bool WALK>
 __global__ void __launch_bounds__(kBlock) coop_kernel(const FwdParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ __align__(8) unsigned long long ring_bar[2];
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kBlock) coop_kernel(const FwdParams P) {
   double* Xs = reinterpret_cast<double*>(smem + fwd_table_smem(H, STREAM ? P.ring_chunk : 0));
   double* AXI = Xs + 2 * H.n_xk * P.n_f;
   double* AXI2 = AXI + H.n_cden * P.n_f;
-  const CoopBuffers B = coop_buffers(H, AXI2 + H.n_cden * P.n_f);
+  const CoopBuffers B = coop_buffers(H, AXI2 + H.n_cden * P.n_f, WALK);
   const TableView T = table_view(smem, H);
   stage_freqs(H, T, P.X, P.n_f, Xs);
   double acc[ENERGY_IN ? 1 : kCoopFreqPerThread][4];
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kBlock) coop_kernel(const FwdParams P) {
   A.n_f = P.n_f;
   const long long n_tiles = (P.n + kCoopSamples - 1) / kCoopSamples;
   for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x)
-    coop_tile<ENERGY_IN, SAVE, STREAM>(H, T, A, tile, Xs, AXI, AXI2, xr_zero, B, acc, R);
+    coop_tile<ENERGY_IN, SAVE, STREAM, WALK>(H, T, A, tile, Xs, AXI, AXI2, xr_zero, B, acc, R);
   if (ENERGY_IN) return;
   double* row = P.partial + (size_t)blockIdx.x * P.n_f * 4;
   for (int f = w, i = 0; f < P.n_f; f += kCoopWarps, ++i)
@@ -324,6 +324,11 @@ int fwd_blocks_per_sm(int dev, size_t smem) {
   return resident_blocks(dev, (const void*)fwd_kernel<E_IN, SAVE, STREAM>, kBlock, smem);
 }
 
+// The form of the small tile's phase 2 (phase2_shared or phase2_nodes, where the measured line is
+// stated); an instance of its own for each, so that neither carries the other's registers and code.  A
+// streamed table, one too large to sit beside the tile, is walked.
+bool coop_walks(const TableHeader& h, int ring_chunk) { return ring_chunk || h.n_pnode >= h.n_cden; }
+
 // How a launch that takes the tile of few samples (coop_tile) stages its table, as fwd_staging; false
 // where it does not take it.  Monte Carlo launches take it up to two 128-sample tiles per SM, where
 // those leave SMs idle and the tile's latency is the launch's: order 4, 16 frequencies, 5000 samples
@@ -335,25 +340,30 @@ int fwd_blocks_per_sm(int dev, size_t smem) {
 bool coop_staging(const tami_diagram* d, int n_f, long long n, bool energy_in, int* ring_chunk, size_t* smem) {
   if (n_f > kCoopMaxFreq || (!energy_in && n > 2LL * kBlock * device_props(d->device).sms)) return false;
   const size_t optin = device_props(d->device).smem_optin;
-  *ring_chunk = staging_mode() != TAMI_STAGING_STREAMED && coop_smem_bytes(d->hdr, n_f, 0) <= optin ? 0 : ring_chunk_ops();
-  *smem = coop_smem_bytes(d->hdr, n_f, *ring_chunk);
+  auto bytes = [&](int chunk) { return coop_smem_bytes(d->hdr, n_f, chunk, coop_walks(d->hdr, chunk)); };
+  *ring_chunk = staging_mode() != TAMI_STAGING_STREAMED && bytes(0) <= optin ? 0 : ring_chunk_ops();
+  *smem = bytes(*ring_chunk);
   return *smem <= optin;
 }
 
 template <bool E_IN, bool SAVE>
-int coop_blocks_per_sm(int dev, int chunk, size_t smem) {
-  return resident_blocks(dev, chunk ? (const void*)coop_kernel<E_IN, SAVE, true> : (const void*)coop_kernel<E_IN, SAVE, false>,
-                         kBlock, smem);
+void (*coop_instance(const tami_diagram* d, int chunk))(const FwdParams) {
+  return chunk ? coop_kernel<E_IN, SAVE, true, true>
+       : coop_walks(d->hdr, chunk) ? coop_kernel<E_IN, SAVE, false, true> : coop_kernel<E_IN, SAVE, false, false>;
+}
+
+template <bool E_IN, bool SAVE>
+int coop_blocks_per_sm(const tami_diagram* d, int chunk, size_t smem) {
+  return resident_blocks(d->device, (const void*)coop_instance<E_IN, SAVE>(d, chunk), kBlock, smem);
 }
 
 template <bool E_IN, bool SAVE>
 int launch_coop(const tami_diagram* d, FwdParams& P, int chunk, size_t smem, cudaStream_t stream, int max_blocks) {
   P.ring_chunk = chunk;
   const long long tiles = (P.n + kCoopSamples - 1) / kCoopSamples;
-  long long grid = std::min(tiles, (long long)device_props(d->device).sms * coop_blocks_per_sm<E_IN, SAVE>(d->device, chunk, smem));
+  long long grid = std::min(tiles, (long long)device_props(d->device).sms * coop_blocks_per_sm<E_IN, SAVE>(d, chunk, smem));
   if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
-  if (chunk) coop_kernel<E_IN, SAVE, true><<<(unsigned)grid, kBlock, smem, stream>>>(P);
-  else coop_kernel<E_IN, SAVE, false><<<(unsigned)grid, kBlock, smem, stream>>>(P);
+  coop_instance<E_IN, SAVE>(d, chunk)<<<(unsigned)grid, kBlock, smem, stream>>>(P);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "coop_kernel launch");
 }
@@ -397,8 +407,8 @@ int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nul
     size_t cs = 0;
     int cc = 0;
     if (coop && coop_staging(d, n_f, n, false, &cc, &cs)) {
-      const int per_sm = std::min(coop_blocks_per_sm<false, false>(d->device, cc, cs),
-                                  coop_blocks_per_sm<false, true>(d->device, cc, cs));
+      const int per_sm = std::min(coop_blocks_per_sm<false, false>(d, cc, cs),
+                                  coop_blocks_per_sm<false, true>(d, cc, cs));
       return (int)std::min((n + kCoopSamples - 1) / kCoopSamples, (long long)dp.sms * per_sm);
     }
   }

@@ -502,9 +502,10 @@ constexpr int kCoopFreqPerThread = kCoopMaxFreq / kCoopWarps;
 template <bool V>
 struct BoolConst { static constexpr bool value = V; };
 
-// Phase 2 of the small tile: phase2_walk's values and sums, bit for bit, node by node.  A block's
-// four warps wait on latency, not on L1: unrolled loops over all nodes, then over all groups, take
-// 3.02 ms with two external frequencies (250 000 rows x 100), the walk 3.12 ms.
+// Phase 2 of the small tile, in two forms with phase2_walk's values and sums, bit for bit.  A trie of
+// fewer products than denominators is taken node by node, in unrolled loops: its values stay in L1 and
+// the walk's words cost more than they save (energy input, order 3, 300 000 rows x 100: 748 us, 784
+// with the other form; the evaluation example, 100 000 x 50: 63 and 65 us).
 template <bool XR_ZERO>
 __device__ __forceinline__ void phase2_nodes(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
                                              int f, const double* Xs, const double* AXI, const double* AXI2,
@@ -536,24 +537,74 @@ __device__ __forceinline__ void phase2_nodes(const TableHeader& H, const TableVi
   vi_out = vi;
 }
 
-struct CoopBuffers {   // each [count][kCoopSamples]
-  double *K, *E, *x, *fv, *rr, *W1, *W, *CB;
-};
-__host__ __device__ __forceinline__ int coop_rows(const TableHeader& h) {
-  return 2 * h.m + h.N + h.n_combo + h.n_fv + h.n_rden + h.n_g1 + h.n_g2 + h.n_cden;
+// A larger trie is walked with the reciprocals in shared memory, [c][thread], over the rows that phase
+// 1 is done with: in per-thread memory the values of the resident threads outgrow what the tiles leave
+// of L1 (energy input, order 4, 100 000 x 64: 537 -> 525 us, 10 000 x 30: 65 -> 60 us; order-4 forward,
+// 5000 x 16: 55 -> 50 us; order 5, 20 000 x 24: 153 -> 146 us; two external frequencies, 250 000 x
+// 100: 3.02 -> 3.01 ms).  re, im: the thread's own columns.
+template <bool XR_ZERO>
+__device__ __forceinline__ void phase2_shared(const TableHeader& H, const TableView& T, const TileArgs& A, int sl,
+                                              int f, const double* Xs, const double* AXI, const double* AXI2,
+                                              const double* CB, const double* W, double* re, double* im,
+                                              double& vr_out, double& vi_out) {
+#pragma unroll 4
+  for (int c = 0; c < H.n_cden; ++c) {
+    const double b = CB[c * kCoopSamples + sl];
+    const double Dr = XR_ZERO ? b : fma(T.cden_a[c], Xs[2 * (T.cden_xk[c] * A.n_f + f)], b);
+    const double r = rcp(fma(Dr, Dr, AXI2[c * A.n_f + f]));
+    re[c * kBlock] = imul(Dr, r);
+    im[c * kBlock] = neg_bits(imul(AXI[c * A.n_f + f], r));
+  }
+  double2 kept[kMaxProdNodes];
+  double vr = H.g2_const ? W[sl] : 0.0, vi = 0.0;
+  double2 run = make_double2(0.0, 0.0);
+  const int* p = T.p2prog;
+#pragma unroll 1
+  for (int hg = H.g2_const; hg < H.n_g2; ++hg) {
+    const double w = W[hg * kCoopSamples + sl];
+    const int e = *p++, src = e & 0xffff;
+    if (src < H.n_cden) run = make_double2(re[src * kBlock], im[src * kBlock]);
+    else if (src != kP2Last) run = kept[src - H.n_cden];
+#pragma unroll 1
+    for (int k = e >> 16; k > 0; --k) {
+      const int x = *p++, slot = x >> 8;
+      const double qr = re[(x & 255) * kBlock], qi = im[(x & 255) * kBlock];
+      run = make_double2(fma(run.x, qr, neg_bits(imul(run.y, qi))), fma(run.x, qi, imul(run.y, qr)));
+      if (slot) kept[slot - H.n_cden] = run;
+    }
+    vr = fma(w, run.x, vr);
+    vi = fma(w, run.y, vi);
+  }
+  vr_out = vr;
+  vi_out = vi;
 }
-__device__ __forceinline__ CoopBuffers coop_buffers(const TableHeader& H, double* p) {
+
+struct CoopBuffers {   // each [count][kCoopSamples]
+  double *K, *E, *x, *fv, *rr, *W1, *W, *CB;   // phase 2: the reciprocals over K .. W1
+};
+// rows of phase 1, or of the reciprocals of kBlock threads (walk: phase2_shared)
+__host__ __device__ __forceinline__ int coop_phase_rows(const TableHeader& h, bool walk) {
+  const int p1 = 2 * h.m + h.N + h.n_combo + h.n_fv + h.n_rden + h.n_g1;
+  const int p2 = walk ? 2 * h.n_cden * kCoopWarps : 0;
+  return p1 > p2 ? p1 : p2;
+}
+__host__ __device__ __forceinline__ int coop_rows(const TableHeader& h, bool walk) {
+  return coop_phase_rows(h, walk) + h.n_g2 + h.n_cden;
+}
+__device__ __forceinline__ CoopBuffers coop_buffers(const TableHeader& H, double* p, bool walk) {
   CoopBuffers B;
   auto take = [&](int rows) { double* q = p; p += rows * kCoopSamples; return q; };
   B.K = take(2 * H.m); B.E = take(H.N); B.x = take(H.n_combo); B.fv = take(H.n_fv); B.rr = take(H.n_rden);
-  B.W1 = take(H.n_g1); B.W = take(H.n_g2); B.CB = take(H.n_cden);
+  B.W1 = take(H.n_g1);
+  p = B.K + coop_phase_rows(H, walk) * kCoopSamples;
+  B.W = take(H.n_g2); B.CB = take(H.n_cden);
   return B;
 }
 
 // Same operations in the same order as fwd_tile, so the same per-sample bits.  STREAM: the program
 // comes through the ring R; a warp steps over the ops of the other warps' groups, since every thread
 // of the block takes part in every move to the next chunk.  Ends with a barrier.
-template <bool ENERGY_IN, bool SAVE, bool STREAM>
+template <bool ENERGY_IN, bool SAVE, bool STREAM, bool WALK>
 __device__ __forceinline__ void coop_tile(const TableHeader& H, const TableView& T, const TileArgs& A, long long tile,
                                           const double* Xs, const double* AXI, const double* AXI2, bool xr_zero,
                                           const CoopBuffers& B, double (*acc)[4], OpRing& R) {
@@ -652,7 +703,11 @@ __device__ __forceinline__ void coop_tile(const TableHeader& H, const TableView&
     constexpr bool XR_ZERO = decltype(zero)::value;
     for (int f = w, i = 0; f < A.n_f; f += kCoopWarps, ++i) {
       double vr, vi;
-      phase2_nodes<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, vr, vi);
+      if (WALK)
+        phase2_shared<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, B.K + threadIdx.x,
+                               B.K + H.n_cden * kBlock + threadIdx.x, vr, vi);
+      else
+        phase2_nodes<XR_ZERO>(H, T, A, sl, f, Xs, AXI, AXI2, B.CB, B.W, vr, vi);
       if (!active) continue;
       if (ENERGY_IN) {
         double2* o = reinterpret_cast<double2*>(A.per_sample) + (size_t)f * A.n + s;

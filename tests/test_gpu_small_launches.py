@@ -52,6 +52,18 @@ def test_small_forward_equals_the_slice_of_a_large_one(order, index, n_f):
         assert torch.all((m - p.mean(dim=1)).abs() <= 1e-13 * scale), n
 
 
+@pytest.mark.parametrize("order,index", [(3, 0), (4, 2), (4, 40), (5, 12), (5, 44)])
+def test_small_forward_off_the_axis(order, index):
+    """Both forms of the small tile's frequency loop (tries of fewer products than denominators, and
+    larger ones) off the imaginary axis, against the 128-sample tile's bits."""
+    D, _ = diagram(order, index)
+    X = W.real_axis(-3.0, 3.0, 7, 0.1)
+    big_n = 3 * 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    _, _, big = D.forward(LAT, 5, 0, big_n, X, 4.0, per_sample=True)
+    for n in (1, 33, 1000):
+        assert torch.equal(D.forward(LAT, 5, 0, n, X, 4.0, per_sample=True)[2], big[:, :n]), n
+
+
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 1000])
 def test_energy_input_equals_the_rows_of_more_frequencies(n):
     """257 frequencies are above the small tile's limit and take the 128-sample one."""
