@@ -330,7 +330,8 @@ int fwd_blocks_per_sm(int dev, size_t smem) {
 bool coop_walks(const TableHeader& h, int ring_chunk) { return ring_chunk || h.n_pnode >= h.n_cden; }
 
 // How a launch that takes the tile of few samples (coop_tile) stages its table, as fwd_staging; false
-// where it does not take it.  Monte Carlo launches take it up to two 128-sample tiles per SM, where
+// where it does not take it.  (What a call refuses is fwd_staging's answer alone, at every n: some
+// tables fit beside this tile's smaller buffers only.)  Monte Carlo launches take it up to two 128-sample tiles per SM, where
 // those leave SMs idle and the tile's latency is the launch's: order 4, 16 frequencies, 5000 samples
 // 114 -> 53 us; order 3, 32 frequencies with per-sample values, 20 000 samples 86 -> 74 us, but
 // 65 537 samples 121 -> 148 us.  Energy input, which keeps no running sums, takes it at every size
@@ -358,22 +359,26 @@ int coop_blocks_per_sm(const tami_diagram* d, int chunk, size_t smem) {
 }
 
 template <bool E_IN, bool SAVE>
-int launch_coop(const tami_diagram* d, FwdParams& P, int chunk, size_t smem, cudaStream_t stream, int max_blocks) {
+int launch_coop(const tami_diagram* d, FwdParams& P, int chunk, size_t smem, cudaStream_t stream, int max_blocks,
+                int* launched) {
   P.ring_chunk = chunk;
   const long long tiles = (P.n + kCoopSamples - 1) / kCoopSamples;
   long long grid = std::min(tiles, (long long)device_props(d->device).sms * coop_blocks_per_sm<E_IN, SAVE>(d, chunk, smem));
   if (max_blocks > 0 && grid > max_blocks) grid = max_blocks;
+  if (launched) *launched = (int)grid;
   coop_instance<E_IN, SAVE>(d, chunk)<<<(unsigned)grid, kBlock, smem, stream>>>(P);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "coop_kernel launch");
 }
 
+// max_blocks: the rows that P.partial holds (0: no partial sums); launched: the blocks that wrote one
 template <bool E_IN, bool SAVE>
-int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max_blocks) {
-  size_t smem = 0;
-  int chunk = 0;
-  if (coop_staging(d, P.n_f, P.n, E_IN, &chunk, &smem)) return launch_coop<E_IN, SAVE>(d, P, chunk, smem, stream, max_blocks);
+int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max_blocks, int* launched = nullptr) {
+  size_t smem = 0, coop_smem = 0;
+  int chunk = 0, coop_chunk = 0;
   if (!fwd_staging(d, P.n_f, &chunk, &smem)) return TAMI_EUNSUPPORTED;
+  if (coop_staging(d, P.n_f, P.n, E_IN, &coop_chunk, &coop_smem))
+    return launch_coop<E_IN, SAVE>(d, P, coop_chunk, coop_smem, stream, max_blocks, launched);
   P.ring_chunk = chunk;
   DeviceProps dp = device_props(d->device);
   const int per_sm = chunk ? fwd_blocks_per_sm<E_IN, SAVE, true>(d->device, smem) : fwd_blocks_per_sm<E_IN, SAVE, false>(d->device, smem);
@@ -619,7 +624,7 @@ int tami_forward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed, 
     P.per_sample = per_sample;
     P.saved = saved;
     P.partial = partial;
-    rc = saved ? launch_fwd<false, true>(d, P, st, grid) : launch_fwd<false, false>(d, P, st, grid);
+    rc = saved ? launch_fwd<false, true>(d, P, st, grid, &used_grid) : launch_fwd<false, false>(d, P, st, grid, &used_grid);
     if (rc) return rc;
   }
   const cudaError_t e = launch_after(finalize_kernel, n_f, kFinBlock, st, partial, used_grid, n_f, n_samples, mean, var);
@@ -662,7 +667,7 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
   P.per_sample = per_sample;
   P.partial = partial;
   jit_mark_generic(const_cast<tami_diagram*>(d));
-  rc = launch_fwd<false, false>(d, P, st, grid);
+  rc = launch_fwd<false, false>(d, P, st, grid, &grid);
   if (rc) return rc;
   const cudaError_t e = launch_after(finalize_kernel, n_f, kFinBlock, st, partial, grid, n_f, n_samples, mean, var);
   return e == cudaSuccess ? TAMI_OK : cuda_fail(e, "finalize launch");
