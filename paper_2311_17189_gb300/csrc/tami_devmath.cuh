@@ -160,7 +160,8 @@ __device__ __forceinline__ double rcp(double d) {
 // point a = j pi/512, |d| <= pi/1024, and
 //   cos phi = C - C (1 - cos d) - S sin d,   sin phi = S - S (1 - cos d) + C sin d
 // with 1 - cos d = d^2/2 - d^4/24 and sin d = d - d^3/6 + d^5/120 (W. J. Cody and W. Waite 1980,
-// reduction and series; truncation below 2e-18).  Values at 2^-61, within 4e-18 of the true ones.
+// reduction and series; truncation below 2e-18).  Values at 2^-61, within 6e-18 of the true ones;
+// the sine within 5 pi/1024 of a multiple of pi comes from sin_near, relatively accurate down to 0.
 // 250 clocks of an SM quarter per warp for a cosine, 1200 with an FP64 Taylor series to r^20; a
 // line energy 373 against 1520, with its gradients 655 against 2580 (order-5 forward, 2^23 samples,
 // one frequency: 9.6 -> 5.6 ms; order-4 forward + adjoint, 2^24 samples x 16 frequencies: 78.6 ->
@@ -296,7 +297,64 @@ __device__ const __align__(16) unsigned long long kTrigTab[514] = {
   0x00648747f37b1e12ull, 0x1fff62169b92db57ull, 0x003243e1fcce00e2ull, 0x1fffd8858e8a924dull,
   0x0000000000000000ull, 0x2000000000000000ull};
 
-struct FixedTrig { long long c, s; };   // cos and sin, times 2^61
+// sin k next to a multiple of pi (|k - n pi| < 2^-6, |k| < 32), within 0.52 ulp, where a fixed-point
+// value keeps no relative accuracy.  r = |k - n pi| is put on 64 significant bits: k's own significand
+// for n = 0, else |k| in turns, |k| 2^58 times 2^134/(2 pi), with 64 bits more than trig_fixed's (a
+// double below 32 is never closer than 1.2e-16 to a multiple of pi); then
+// sin r = r (1 - r^2/6 + r^4/120 - r^6/5040).  One argument in a hundred comes here, a warp in four for
+// one of its lanes: out of line, and in integers, as FP64 instructions would take as long as the whole
+// fixed-point sine.
+static __device__ __noinline__ double sin_near(double k) {
+  const unsigned int hi = (unsigned int)__double2hiint(k);
+  const int ek = (int)(hi >> 20) & 0x7FF;
+  if (ek < 990) return k;                                                            // |k| < 2^-33
+  unsigned int sign = hi & 0x80000000u;
+  unsigned long long m = (((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | (unsigned int)__double2loint(k)) << 11;
+  int e = ek - 1023;                                                                 // |k| = m 2^(e - 63)
+  if (e >= 0) {
+    const unsigned long long K = m >> (5 - e);                                       // |k| 2^58
+    const unsigned int kl = (unsigned int)K, kh = (unsigned int)(K >> 32);
+    const unsigned long long t0 = (unsigned long long)kl * 0xE441529Fu;
+    const unsigned long long t1 = (unsigned long long)kh * 0xE441529Fu + (t0 >> 32);
+    const unsigned long long t2 = (unsigned long long)kl * 0x2F9836E4u + (unsigned int)t1;
+    const unsigned long long low = mulhi_trunc(K, 0x613ABE8FA9A6EE06ull) << 1;
+    unsigned long long tl = ((t2 << 32) | (unsigned int)t0) + low;
+    unsigned long long th = K * 10ull + (unsigned long long)kh * 0x2F9836E4u + (t1 >> 32) + (t2 >> 32) + (tl < low ? 1u : 0u);
+    const bool odd = (long long)th < 0;                                              // half turns, |k| = (odd + (th, tl) 2^-128) pi
+    th = (th << 1) | (tl >> 63);
+    tl <<= 1;
+    const bool under = (long long)th < 0;                                            // from the next multiple down
+    if (under) {
+      th = ~th + (tl == 0ull ? 1u : 0u);
+      tl = 0ull - tl;
+    }
+    sign ^= odd ? 0x80000000u : 0u;   // (-1)^n and r's sign: n is odd + 1 where r is below 0, and the two cancel
+    const int z = min(max(__clzll((long long)th), 1), 63);
+    m = mulhi_trunc(((th << z) | (tl >> (64 - z))) >> 1, 0x6487ED5110B4611Aull) << 2;   // times pi 2^-2
+    e = 1 - z;
+    if (!(m >> 63)) { m <<= 1; --e; }
+  }
+  const unsigned long long rf = m >> min(-5 - e, 63);                                // r 2^68
+  const unsigned long long r2 = mulhi_trunc(rf, rf);                                 // r^2 2^72
+  const unsigned int r2h = (unsigned int)(r2 >> 28);                                 // r^2 2^44
+  const unsigned int q = __umulhi(r2h, 2290649225u - __umulhi(r2h, 13315u));         // (r^2/120 - r^4/5040) 2^50
+  const unsigned long long c = mulhi_trunc(r2, 0x2AAAAAAAAAAAAAABull - ((unsigned long long)q << 14));   // 1 - sin(r)/r, 2^72
+  m -= mulhi_trunc(m >> 1, c) >> 7;
+  if (!(m >> 63)) { m <<= 1; --e; }
+  return pack62(m >> 1, e + 1023, sign);
+}
+
+struct FixedTrig { long long c; double s; };   // cos times 2^61, sin
+
+// v 2^-S rounded to the nearest double
+template <int S>
+__device__ __forceinline__ double fixed_to_double(long long v) {
+  const unsigned int sign = (unsigned int)(v >> 32) & 0x80000000u;
+  const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+  const int z = __clzll((long long)m);
+  const double r = pack62((m << (z & 63)) >> 1, 1086 - S - z, sign);
+  return m == 0ull ? 0.0 : r;
+}
 
 // |k| < 32 (larger arguments, infinities and NaNs take the FP64 path); NEED_SIN = false leaves s out
 template <bool NEED_SIN>
@@ -320,8 +378,8 @@ __device__ __forceinline__ FixedTrig trig_fixed(double k) {
   const unsigned int x4 = __umulhi(x2h, x2h);                                       // d^4 2^64
   const unsigned long long cm = x2 - ((unsigned long long)__umulhi(x4, 178956971u) << 15);   // (1 - cos d) 2^79
   const unsigned int x3 = __umulhi(x2h, (unsigned int)(x >> 29));                   // d^3 2^56
-  const unsigned int w = 715827883u - __umulhi(x2h, 546u);                     // (1/6 - d^2/120) 2^32
-  const unsigned long long sd = x - ((unsigned long long)__umulhi(x3, w) << 13);    // |sin d| 2^69
+  const unsigned int w = 2863311531u - __umulhi(x2h, 2185u);                        // (1/6 - d^2/120) 2^34
+  const unsigned long long sd = x - (((2ull * x3 + min(x3, 1u)) * w) >> 22);        // |sin d| 2^69, x3's middle
   const ulonglong2 cs = __ldg(reinterpret_cast<const ulonglong2*>(kTrigTab) + j);
   const unsigned long long sdn = sd << 2;                                           // 2^71
   const long long Ss = (long long)(mulhi_trunc(cs.y, sdn) >> 7);                    // S |sin d| 2^61
@@ -329,48 +387,51 @@ __device__ __forceinline__ FixedTrig trig_fixed(double k) {
   c = neg ? c + Ss : c - Ss;
   FixedTrig r;
   r.c = (q + 1u) & 2u ? -c : c;
-  r.s = 0;
+  r.s = 0.0;
   if (NEED_SIN) {
     const long long Cs = (long long)(mulhi_trunc(cs.x, sdn) >> 7);
     long long v = (long long)(cs.y - (mulhi_trunc(cs.y, cm) >> 15));
     v = neg ? v - Cs : v + Cs;
-    r.s = ((q >> 1) ^ (hi >> 31)) & 1u ? -v : v;
+    r.s = j <= 2u ? sin_near(k) : fixed_to_double<61>(((q >> 1) ^ (hi >> 31)) & 1u ? -v : v);
   }
   return r;
 }
 
-// v 2^-S rounded to the nearest double
-template <int S>
-__device__ __forceinline__ double fixed_to_double(long long v) {
-  const unsigned int sign = (unsigned int)(v >> 32) & 0x80000000u;
-  const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
-  const int z = __clzll((long long)m);
-  const double r = pack62((m << (z & 63)) >> 1, 1086 - S - z, sign);
-  return m == 0ull ? 0.0 : r;
+// Arguments of 32 and above, infinities and NaNs: r = k - n pi on the FP64 unit with pi in three parts
+// (a NaN for infinities and NaNs; from about 2^53 on the remainder of 2 pi's nearest double), and
+// whether n is odd, which flips both signs.
+__device__ __forceinline__ bool trig_far(double k) { return (__double2hiint(k) & 0x7FF00000) > 0x40300000; }
+__device__ __forceinline__ double trig_reduce(double k, bool& odd) {
+  const double n = rint(k * 0x1.45f306dc9c883p-2);
+  double r = fma(-n, 0x1.921fb54442d18p+1, k);
+  r = fma(-n, 0x1.1a62633145c07p-53, r);
+  r = fma(-n, -0x1.f1976b7ed8fbcp-109, r);
+  const bool good = fabs(r) <= 2.0;
+  odd = good && ((long long)n & 1) != 0;
+  return good ? r : fmod(k, 0x1.921fb54442d18p+2);
 }
 
-// Arguments of 32 and above, infinities and NaNs: reduced on the FP64 unit by 2 pi in three parts,
-// out of line (a NaN for infinities and NaNs).
-__device__ __forceinline__ bool trig_far(double k) { return (__double2hiint(k) & 0x7FF00000) > 0x40300000; }
-__device__ __forceinline__ double trig_reduce(double k) {
-  const double n = rint(k * 0x1.45f306dc9c883p-3);
-  double r = fma(-n, 0x1.921fb54442d18p+2, k);
-  r = fma(-n, 0x1.1a62633145c07p-52, r);
-  r = fma(-n, -0x1.f1976b7ed8fbcp-108, r);
-  return fabs(r) <= 8.0 ? r : fmod(k, 0x1.921fb54442d18p+2);
+template <bool NEED_SIN>
+__device__ __forceinline__ FixedTrig trig_any(double k, bool& finite) {
+  bool odd = false;
+  const double r = trig_far(k) ? trig_reduce(k, odd) : k;
+  FixedTrig t = trig_fixed<NEED_SIN>(r);
+  if (odd) { t.c = -t.c; t.s = -t.s; }
+  finite = r == r;
+  return t;
 }
 
 __device__ __forceinline__ double cw_cos(double k) {
-  const double r = trig_far(k) ? trig_reduce(k) : k;
-  const double c = fixed_to_double<61>(trig_fixed<false>(r).c);
-  return r == r ? c : r;
+  bool finite;
+  const double c = fixed_to_double<61>(trig_any<false>(k, finite).c);
+  return finite ? c : k - k;
 }
 
 __device__ __forceinline__ void cw_sincos(double k, double& s_out, double& c_out) {
-  const double r = trig_far(k) ? trig_reduce(k) : k;
-  const FixedTrig t = trig_fixed<true>(r);
-  s_out = r == r ? fixed_to_double<61>(t.s) : r;
-  c_out = r == r ? fixed_to_double<61>(t.c) : r;
+  bool finite;
+  const FixedTrig t = trig_any<true>(k, finite);
+  s_out = finite ? t.s : k - k;
+  c_out = finite ? fixed_to_double<61>(t.c) : k - k;
 }
 
 // E = mu - eps(k),  eps(k) = -2t(cos kx + cos ky) - 4t' cos kx cos ky, from the fixed-point cosines:
@@ -384,12 +445,11 @@ __device__ __forceinline__ double line_energy_of(long long cx, long long cy, dou
 }
 
 template <bool GRAD>
-__device__ __forceinline__ double line_energy_near(double kx, double ky, double t, double tp, double mu, double& gx,
-                                                   double& gy) {
-  const FixedTrig x = trig_fixed<GRAD>(kx), y = trig_fixed<GRAD>(ky);
+__device__ __forceinline__ double line_energy_from(const FixedTrig& x, const FixedTrig& y, double t, double tp, double mu,
+                                                   double& gx, double& gy) {
   if (GRAD) {
-    gx = fma(4.0 * tp, fixed_to_double<61>(y.c), 2.0 * t) * fixed_to_double<61>(x.s);
-    gy = fma(4.0 * tp, fixed_to_double<61>(x.c), 2.0 * t) * fixed_to_double<61>(y.s);
+    gx = fma(4.0 * tp, fixed_to_double<61>(y.c), 2.0 * t) * x.s;
+    gy = fma(4.0 * tp, fixed_to_double<61>(x.c), 2.0 * t) * y.s;
   }
   return line_energy_of(x.c, y.c, t, tp, mu);
 }
@@ -399,9 +459,10 @@ __device__ __forceinline__ double line_energy_near(double kx, double ky, double 
 template <bool GRAD>
 static __device__ __noinline__ double line_energy_far(double kx, double ky, double t, double tp, double mu, double& gx,
                                                       double& gy) {
-  const double rx = trig_far(kx) ? trig_reduce(kx) : kx, ry = trig_far(ky) ? trig_reduce(ky) : ky;
-  const double E = line_energy_near<GRAD>(rx, ry, t, tp, mu, gx, gy);
-  const double bad = (rx - rx) + (ry - ry);          // 0, or a NaN
+  bool fx, fy;
+  const FixedTrig x = trig_any<GRAD>(kx, fx), y = trig_any<GRAD>(ky, fy);
+  const double E = line_energy_from<GRAD>(x, y, t, tp, mu, gx, gy);
+  const double bad = fx && fy ? 0.0 : (kx - kx) + (ky - ky);          // 0, or a NaN
   if (GRAD) { gx += bad; gy += bad; }
   return E + bad;
 }
@@ -412,7 +473,7 @@ static __device__ __noinline__ double line_energy_far(double kx, double ky, doub
 __device__ TAMI_LINE_INLINE double line_energy(double kx, double ky, double t, double tp, double mu) {
   double gx, gy;
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<false>(kx, ky, t, tp, mu, gx, gy);
-  return line_energy_near<false>(kx, ky, t, tp, mu, gx, gy);
+  return line_energy_from<false>(trig_fixed<false>(kx), trig_fixed<false>(ky), t, tp, mu, gx, gy);
 }
 
 // Energy of a line that carries k_ext, with the factors G = (2t + 4t' cos K_perp) sin K of
@@ -420,7 +481,7 @@ __device__ TAMI_LINE_INLINE double line_energy(double kx, double ky, double t, d
 __device__ TAMI_LINE_INLINE double line_energy_grad(double kx, double ky, double t, double tp, double mu, double& gx,
                                                    double& gy) {
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<true>(kx, ky, t, tp, mu, gx, gy);
-  return line_energy_near<true>(kx, ky, t, tp, mu, gx, gy);
+  return line_energy_from<true>(trig_fixed<true>(kx), trig_fixed<true>(ky), t, tp, mu, gx, gy);
 }
 
 // e^t and e^t - 1 for t <= 0 in fixed point, after P. T. P. Tang, "Table-driven implementation of the
