@@ -211,9 +211,9 @@ __global__ void exp_selftest_kernel(const double* t, long long n, double* y, dou
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double e = 0.0;
-  y[i] = exp_neg<true>(t[i], e);
+  y[i] = exp_neg<kBoseExp>(t[i], e);
   em[i] = e;
-  if (y_plain) y_plain[i] = exp_neg<false>(t[i], e);
+  if (y_plain) y_plain[i] = exp_neg<kFermiExp>(t[i], e);
 }
 
 __global__ void sincos_selftest_kernel(const double* k, long long n, double* s, double* c) {

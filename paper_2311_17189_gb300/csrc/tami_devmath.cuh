@@ -494,7 +494,9 @@ __device__ TAMI_LINE_INLINE double line_energy_grad(double kx, double ky, double
 // on t's own significand, so the result is relatively exact down to t = 0.  190 clocks of an SM
 // quarter per warp for e^t, 250 with e^t - 1; an FP64 polynomial after a 256-entry table took 859
 // and 1102 (order-5 forward, 2^23 samples, one frequency: 13.3 -> 9.6 ms).  Within 0.51 ulp, e^t - 1
-// within 0.75; e^t below 2^-1022 is 0.
+// within 0.75; e^t below 2^-1022 is rounded to a subnormal value with kExpSubnormal, else 0 (for code
+// whose products flush those anyway).
+constexpr int kExpMinusOne = 1, kExpSubnormal = 2, kFermiExp = kExpSubnormal, kBoseExp = kExpSubnormal | kExpMinusOne;
 __device__ const __align__(16) unsigned long long kExpTab[1024] = {
   0x0000000000000000ull, 0x002c58ae3f081ef4ull, 0x0058a9ade372512eull, 0x0084f30041ea698bull,
   0x00b134a6aee1375bull, 0x00dd6ea27e8c909dull, 0x0109a0f504e75c36ull, 0x0135cb9f95b19c24ull,
@@ -753,8 +755,9 @@ __device__ const __align__(16) unsigned long long kExpTab[1024] = {
   0x7f4e12b026665494ull, 0x7f645dd9b2525896ull, 0x7f7aa5269a17747cull, 0x7f90e89788f85850ull,
   0x7fa7282d2a1a094full, 0x7fbd63e82883e713ull, 0x7fd39bc92f1fb0afull, 0x7fe9cfd0e8b989d8ull};
 
-template <bool NEED_EM>
+template <int FORM>
 __device__ __forceinline__ double exp_neg(double t, double& em) {
+  constexpr bool NEED_EM = (FORM & kExpMinusOne) != 0;
   const unsigned int hi = (unsigned int)__double2hiint(t) & 0x7FFFFFFFu, lo = (unsigned int)__double2loint(t);
   const int et = (int)(hi >> 20);
   const unsigned long long M = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
@@ -786,7 +789,9 @@ __device__ __forceinline__ double exp_neg(double t, double& em) {
   const double r = pack62(y, ey, 0u);
   const bool big = hi >= 0x40900000u;                                                         // |t| >= 1024, NaN
   const bool nan = hi > 0x7FF00000u || (hi == 0x7FF00000u && lo != 0u);
-  const double tail = nan ? t : 0.0;                                                          // e^t below 2^-1022: 0
+  double tail = nan ? t : 0.0;                                                                // e^t below 2^-1022
+  if ((FORM & kExpSubnormal) && ey < 1 && ey > -53 && !big)                                   // y 2^(ey - 11) of 2^-1074
+    tail = __longlong_as_double((long long)((y + (1ull << (10 - ey))) >> (11 - ey)));
   if (NEED_EM) {
     // 1 - e^t: leading bit at 2^63 after the shift, exponent e1 of that bit
     const unsigned long long D1 = 0ull - (((0ull - D0) >> min(I, 63)) | 1ull);
@@ -846,7 +851,7 @@ __device__ __forceinline__ void fermi_segment(const int* seg, const int* fvr, co
                                               double* fv, double* fvd) {
   const double xv = x[seg[0] * S];
   double em = 0.0;
-  const double y = exp_neg<BOSE>(neg_bits(imul(beta, fabs(xv))), em);
+  const double y = exp_neg<BOSE ? kBoseExp : kFermiExp>(neg_bits(imul(beta, fabs(xv))), em);
   const double rD = rcp(BOSE ? neg_bits(em) : 1.0 + y);
   const double t2 = imul(BOSE ? neg_bits(y) : y, rD);
   const bool neg = __double_as_longlong(xv) <= 0;   // xv <= 0 (+0, -0 and negatives), on the ALU

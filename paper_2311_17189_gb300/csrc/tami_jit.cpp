@@ -231,6 +231,7 @@ bool keep_rr() {
 // order 5 6.99 against 6.42 ms): there the integer product's registers cost more than its slots.
 // $TAMI_JIT_PSMUL=0 keeps every product on the FP64 unit, =all moves every one, =fwd every one of
 // the forward part.
+bool flushes(const TableHeader& h, int kind) { return kind != kKindEnergy && h.n_ops <= 256; }
 struct PsShare { double fwd = 1.0, rev = 1.0; };
 PsShare ps_share(PsShare balanced) {
   const char* e = std::getenv("TAMI_JIT_PSMUL");
@@ -578,11 +579,13 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     o("__device__ const double kJitXvec[%d] = {%s};", h.n_xk * h.n_ext, v.c_str());
   }
   {
-    // one out-of-line copy of a Fermi segment's exponential, reciprocal and selects
+    // one out-of-line copy of a Fermi segment's exponential, reciprocal and selects; subnormal values of
+    // e^t only where the products keep them (flushes)
+    const bool sub = !flushes(h, kind);
     for (int bose = 0; bose < 2; ++bose) {
       o("static __device__ __noinline__ double2 tami_seg_%s(double xv, double beta) {", bose ? "bose" : "fermi");
       o("  double em = 0.0;");
-      o("  const double y = exp_neg<%s>(%s, em); (void)em;", bose ? "true" : "false", PM("-beta", "fabs(xv)").c_str());
+      o("  const double y = exp_neg<%s>(%s, em); (void)em;", bose ? (sub ? "kBoseExp" : "true") : (sub ? "kFermiExp" : "false"), PM("-beta", "fabs(xv)").c_str());
       o("  const double rD = rcp(%s);", bose ? "-em" : "1.0 + y");
       o("  const double t2 = %s;", PM(bose ? "(-y)" : "(y)", "rD").c_str());
       o("  const bool neg = __double_as_longlong(xv) <= 0;");
