@@ -182,7 +182,10 @@ int tami_sample_energies(const tami_diagram* d, const tami_lattice* lat, uint64_
 int tami_eval_energies(const tami_diagram* d, const double* E, int64_t n_e, const double* X, int n_f,
                        double beta, double* out, tami_stream_t stream);
 
-/* Scratch needed by tami_forward for n samples and n_f frequencies (per-block partial sums). */
+/* Scratch needed by tami_forward for up to n samples and n_f frequencies (per-block partial sums): a
+ * workspace queried for n serves every smaller call at n_f.  A call refuses less than one row of
+ * sums per 128 samples (up to the blocks that fit the GPU); between that and the queried size its
+ * sums are grouped into as many rows as there are. */
 int tami_forward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, size_t* bytes);
 
 /* Monte Carlo evaluation over momenta (Sec. 5.2; samples and their energies as in
@@ -197,13 +200,14 @@ int tami_forward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, si
  *               momenta, energies and trig (term products are still recomputed).  Row-major,
  *               sample index fastest.
  *   workspace   device, at least tami_forward_workspace() bytes, 256-byte aligned.
- * The reduction is deterministic for fixed (n, n_f, device). */
+ * The reduction is deterministic for fixed (n, n_f, device) and a workspace of at least the size
+ * queried for n. */
 int tami_forward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed, uint64_t offset,
                  int64_t n_samples, const double* X, int n_f, double beta, double* mean, double* var,
                  double* per_sample, double* saved, void* workspace, size_t workspace_bytes,
                  tami_stream_t stream);
 
-/* Scratch needed by tami_backward for n samples and n_f frequencies. */
+/* Scratch needed by tami_backward for up to n samples and n_f frequencies (as tami_forward_workspace). */
 int tami_backward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, size_t* bytes);
 
 /* Adjoint of tami_forward's mean (the paper defines only the forward evaluation, Sec. 2.3 and
@@ -231,7 +235,8 @@ int tami_backward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed,
                   double* per_sample_grads, const double* saved, void* workspace, size_t workspace_bytes,
                   tami_stream_t stream);
 
-/* Scratch needed by tami_forward_backward (per-block partial sums of the adjoint and the forward). */
+/* Scratch needed by tami_forward_backward (per-block partial sums of the adjoint and the forward; as
+ * tami_forward_workspace). */
 int tami_forward_backward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, size_t* bytes);
 
 /* Forward and adjoint in one pass over the samples, for an upstream gradient known beforehand

@@ -495,17 +495,22 @@ bool bwd_generic_ok(const tami_diagram* d, int n_f, bool fwd) {
 // threads (order 3, 5000 samples x 200 frequencies 1605 -> 316 us with 8 lanes, 375 with 16; three
 // bubbles, 20 000 x 100, 1133 -> 403 us with 4; five bubbles, 50 000 x 40, 688 -> 524 us with 2; order
 // 4, 20 000 x 16, 399 -> 322 us; but order 5, 10 000 x 4, 303 -> 367 us: a lane with one frequency).
+constexpr int kBwMostLanes = 3;                            // log2
+long long bwd_lane_samples(int dev, int lq) { return (6LL * kBlock * device_props(dev).sms) >> lq; }   // the most
 int bwd_lanes(const tami_diagram* d, int n_f, long long n) {
-  const long long threads = 6LL * kBlock * device_props(d->device).sms;
   int lq = 0;
-  while (lq < 3 && (8 << lq) <= n_f && n <= (threads >> (lq + 1))) ++lq;
+  while (lq < kBwMostLanes && (8 << lq) <= n_f && n <= bwd_lane_samples(d->device, lq + 1)) ++lq;
   return lq;
 }
 
 // Grid of an adjoint launch (the workspace holds its partial rows).  A table the generic kernel
 // cannot take (*generic_ok = false) runs only on the specialised kernel, whose launch is clamped to
-// the workspace's rows: 4 blocks per SM.
-int bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool fwd, bool* generic_ok = nullptr) {
+// the workspace's rows: 4 blocks per SM.  least: the rows that a call asks of its workspace, one lane a
+// sample; with fewer than the grid's (a workspace queried for more frequencies, say) the grid is cut
+// to them, and only the grouping of the sums depends on it.  most: the rows of a queried workspace, at
+// least the grid of every call of up to n samples.
+struct BwdGrid { int grid, least, most; };
+BwdGrid bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool fwd, bool* generic_ok = nullptr) {
   DeviceProps dp = device_props(d->device);
   const size_t smem = bwd_smem_bytes(d->hdr, n_f, fwd);
   if (smem_out) *smem_out = smem;
@@ -513,19 +518,24 @@ int bwd_grid(const tami_diagram* d, int n_f, long long n, size_t* smem_out, bool
   if (generic_ok) *generic_ok = ok;
   if (!ok) {
     const long long tiles = (n + kBlock - 1) / kBlock;
-    return (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
+    const int grid = (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
+    return {grid, grid, grid};
   }
   auto resident = [&](const void* kernel) { return resident_blocks(d->device, kernel, kBlock, smem); };
   // one grid for both adjoint instances (saved rows or recomputation), so that their reductions
   // group the samples alike and the results agree bit for bit
   const int per_sm = fwd ? resident((const void*)bwd_kernel<false, true>)
                          : std::min(resident((const void*)bwd_kernel<false, false>), resident((const void*)bwd_kernel<true, false>));
-  const int per_tile = kBlock >> bwd_lanes(d, n_f, n);
-  long long tiles = (n + per_tile - 1) / per_tile;
-  long long grid = (long long)dp.sms * per_sm;
-  if (grid > tiles) grid = tiles;
-  if (grid < 1) grid = 1;
-  return (int)grid;
+  auto blocks = [&](long long samples, int lq) {
+    const int per_tile = kBlock >> lq;
+    return (int)std::max(1LL, std::min((samples + per_tile - 1) / per_tile, (long long)dp.sms * per_sm));
+  };
+  BwdGrid g;
+  g.least = g.most = blocks(n, 0);
+  for (int lq = 1; lq <= kBwMostLanes && (4 << lq) <= n_f; ++lq)
+    g.most = std::max(g.most, blocks(std::min(n, bwd_lane_samples(d->device, lq)), lq));
+  g.grid = blocks(n, bwd_lanes(d, n_f, n));
+  return g;
 }
 
 // The fused pass's final reduction: block f < n_f sums dv/dX_f and the forward's four sums of f,
@@ -593,8 +603,8 @@ int tami_backward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, s
   int rc = bwd_check(d, n_f);
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
-  const int grid = bwd_grid(d, n_f, n_samples, nullptr, false);
-  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
+  const int rows = bwd_grid(d, n_f, n_samples, nullptr, false).most;
+  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)rows;
   return TAMI_OK;
 }
 
@@ -602,8 +612,8 @@ int tami_forward_backward_workspace(const tami_diagram* d, int64_t n_samples, in
   int rc = bwd_check(d, n_f);
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
-  const int grid = bwd_grid(d, n_f, n_samples, nullptr, true);
-  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
+  const int rows = bwd_grid(d, n_f, n_samples, nullptr, true).most;
+  *bytes = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)rows;
   return TAMI_OK;
 }
 
@@ -620,10 +630,11 @@ int tami_backward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed,
   if (((uintptr_t)workspace & 255) != 0) { set_error("workspace must be 256-byte aligned"); return TAMI_EINVAL; }
   size_t smem = 0;
   bool generic_ok = true;
-  const int grid = bwd_grid(d, n_f, n_samples, &smem, false, &generic_ok);
+  const BwdGrid g = bwd_grid(d, n_f, n_samples, &smem, false, &generic_ok);
   const std::string generic_why = generic_ok ? std::string() : std::string(tami_last_error());
-  const size_t need = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, false) * (size_t)grid;
-  if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
+  const size_t row = sizeof(double) * (size_t)bwd_nval(n_f, false);
+  if (workspace_bytes < kBwHeadBytes + row * (size_t)g.least) { set_error("workspace too small"); return TAMI_EINVAL; }
+  const int grid = (int)std::min((size_t)g.grid, (workspace_bytes - kBwHeadBytes) / row);
   tami_diagram* dm = const_cast<tami_diagram*>(d);
   const int sel = jit_select(dm, kJitKindBwd, n_samples, n_f, generic_ok);
   if (sel < 0) return -sel;
@@ -674,10 +685,11 @@ int tami_forward_backward(const tami_diagram* d, const tami_lattice* lat, uint64
   if (((uintptr_t)workspace & 255) != 0) { set_error("workspace must be 256-byte aligned"); return TAMI_EINVAL; }
   size_t smem = 0;
   bool generic_ok = true;
-  const int grid = bwd_grid(d, n_f, n_samples, &smem, true, &generic_ok);
+  const BwdGrid g = bwd_grid(d, n_f, n_samples, &smem, true, &generic_ok);
   const std::string generic_why = generic_ok ? std::string() : std::string(tami_last_error());
-  const size_t need = kBwHeadBytes + sizeof(double) * (size_t)bwd_nval(n_f, true) * (size_t)grid;
-  if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
+  const size_t row = sizeof(double) * (size_t)bwd_nval(n_f, true);
+  if (workspace_bytes < kBwHeadBytes + row * (size_t)g.least) { set_error("workspace too small"); return TAMI_EINVAL; }
+  const int grid = (int)std::min((size_t)g.grid, (workspace_bytes - kBwHeadBytes) / row);
   // the diagram's specialised kernel (compiled once and cached with it) or the generic one
   tami_diagram* dm = const_cast<tami_diagram*>(d);
   const int sel = jit_select(dm, kJitKindFused, n_samples, n_f, generic_ok);

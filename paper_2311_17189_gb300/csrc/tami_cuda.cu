@@ -329,8 +329,20 @@ int fwd_blocks_per_sm(int dev, size_t smem) {
 // streamed table, one too large to sit beside the tile, is walked.
 bool coop_walks(const TableHeader& h, int ring_chunk) { return ring_chunk || h.n_pnode >= h.n_cden; }
 
-// How a launch that takes the tile of few samples (coop_tile) stages its table, as fwd_staging; false
-// where it does not take it.  (What a call refuses is fwd_staging's answer alone, at every n: some
+// The most samples of a Monte Carlo launch that may take the tile of few samples.
+long long coop_most_samples(int dev) { return 2LL * kBlock * device_props(dev).sms; }
+
+// How the tile of few samples (coop_tile) stages a table, as fwd_staging; false where it cannot.
+bool coop_fits(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem) {
+  if (n_f > kCoopMaxFreq) return false;
+  const size_t optin = device_props(d->device).smem_optin;
+  auto bytes = [&](int chunk) { return coop_smem_bytes(d->hdr, n_f, chunk, coop_walks(d->hdr, chunk)); };
+  *ring_chunk = staging_mode() != TAMI_STAGING_STREAMED && bytes(0) <= optin ? 0 : ring_chunk_ops();
+  *smem = bytes(*ring_chunk);
+  return *smem <= optin;
+}
+
+// Whether a launch takes the tile of few samples, and how it stages its table.  (What a call refuses is fwd_staging's answer alone, at every n: some
 // tables fit beside this tile's smaller buffers only.)  Monte Carlo launches take it up to two 128-sample tiles per SM, where
 // those leave SMs idle and the tile's latency is the launch's: order 4, 16 frequencies, 5000 samples
 // 114 -> 53 us; order 3, 32 frequencies with per-sample values, 20 000 samples 86 -> 74 us, but
@@ -339,12 +351,8 @@ bool coop_walks(const TableHeader& h, int ring_chunk) { return ring_chunk || h.n
 // us; order 3, 300 000 x 100, 908 -> 755 us; two external frequencies, 250 000 x 100, 3.41 -> 3.02 ms).
 // Above kCoopMaxFreq frequencies a thread's running sums would not fit.
 bool coop_staging(const tami_diagram* d, int n_f, long long n, bool energy_in, int* ring_chunk, size_t* smem) {
-  if (n_f > kCoopMaxFreq || (!energy_in && n > 2LL * kBlock * device_props(d->device).sms)) return false;
-  const size_t optin = device_props(d->device).smem_optin;
-  auto bytes = [&](int chunk) { return coop_smem_bytes(d->hdr, n_f, chunk, coop_walks(d->hdr, chunk)); };
-  *ring_chunk = staging_mode() != TAMI_STAGING_STREAMED && bytes(0) <= optin ? 0 : ring_chunk_ops();
-  *smem = bytes(*ring_chunk);
-  return *smem <= optin;
+  if (!energy_in && n > coop_most_samples(d->device)) return false;
+  return coop_fits(d, n_f, ring_chunk, smem);
 }
 
 template <bool E_IN, bool SAVE>
@@ -394,37 +402,50 @@ int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max
   return TAMI_OK;
 }
 
-// Grid of a momentum-mode forward launch (the workspace holds one partial row per block).  When
-// the generic kernel cannot stage the table (*generic_ok = false) only the specialised kernel can
-// run it, whose launch is clamped to the rows of the workspace: 4 blocks per SM.
-int grid_for(const tami_diagram* d, int n_f, long long n, bool* generic_ok = nullptr, bool coop = true) {
-  DeviceProps dp = device_props(d->device);
+// Grids of a momentum-mode forward launch, whose workspace holds one partial row per block.  The
+// saving instances share the grid of the others (one workspace size for both).
+int tile_grid(const tami_diagram* d, int chunk, size_t smem, long long n) {   // the 128-sample tile
+  const int dev = d->device;
+  const int per_sm = chunk ? std::min(fwd_blocks_per_sm<false, false, true>(dev, smem), fwd_blocks_per_sm<false, true, true>(dev, smem))
+                           : std::min(fwd_blocks_per_sm<false, false, false>(dev, smem), fwd_blocks_per_sm<false, true, false>(dev, smem));
+  return (int)std::max(1LL, std::min((n + kBlock - 1) / kBlock, (long long)device_props(dev).sms * per_sm));
+}
+int coop_grid(const tami_diagram* d, int chunk, size_t smem, long long n) {   // the tile of few samples
+  const int per_sm = std::min(coop_blocks_per_sm<false, false>(d, chunk, smem), coop_blocks_per_sm<false, true>(d, chunk, smem));
+  return (int)std::max(1LL, std::min((n + kCoopSamples - 1) / kCoopSamples, (long long)device_props(d->device).sms * per_sm));
+}
+
+// Blocks of a launch.  Where the generic kernel cannot stage the table (*generic_ok = false) only the
+// specialised kernel can run it, whose launch is clamped to the rows of the workspace: 4 blocks per SM.
+int fwd_grid(const tami_diagram* d, int n_f, long long n, bool* generic_ok) {
+  size_t smem = 0;
+  int chunk = 0, coop_chunk = 0;
+  size_t coop_smem = 0;
+  *generic_ok = fwd_staging(d, n_f, &chunk, &smem);
+  if (!*generic_ok) return (int)std::max(1LL, std::min((n + kBlock - 1) / kBlock, 4LL * device_props(d->device).sms));
+  if (coop_staging(d, n_f, n, false, &coop_chunk, &coop_smem)) return coop_grid(d, coop_chunk, coop_smem, n);
+  return tile_grid(d, chunk, smem, n);
+}
+// Rows that a call asks of its workspace: the 128-sample tile's blocks, with the shared memory that the
+// limits count.  A workspace with fewer rows than fwd_grid (one queried for more frequencies, say)
+// cuts the grid to them, and only the grouping of the sums depends on it.
+int fwd_least_rows(const tami_diagram* d, int n_f, long long n) {
   size_t smem = 0, counted = 0;
   int chunk = 0;
-  const bool ok = fwd_staging(d, n_f, &chunk, &smem, &counted);
-  if (!coop) smem = counted;   // the fixed array's limit
-  if (generic_ok) *generic_ok = ok;
-  if (!ok) {
-    const long long tiles = (n + kBlock - 1) / kBlock;
-    return (int)std::max(1LL, std::min(tiles, 4LL * dp.sms));
-  }
-  {
-    size_t cs = 0;
-    int cc = 0;
-    if (coop && coop_staging(d, n_f, n, false, &cc, &cs)) {
-      const int per_sm = std::min(coop_blocks_per_sm<false, false>(d, cc, cs),
-                                  coop_blocks_per_sm<false, true>(d, cc, cs));
-      return (int)std::min((n + kCoopSamples - 1) / kCoopSamples, (long long)dp.sms * per_sm);
-    }
-  }
-  // the saving instance shares the grid (one workspace size for both)
-  const int per_sm = chunk ? std::min(fwd_blocks_per_sm<false, false, true>(d->device, smem), fwd_blocks_per_sm<false, true, true>(d->device, smem))
-                           : std::min(fwd_blocks_per_sm<false, false, false>(d->device, smem), fwd_blocks_per_sm<false, true, false>(d->device, smem));
-  long long tiles = (n + kBlock - 1) / kBlock;
-  long long grid = (long long)dp.sms * per_sm;
-  if (grid > tiles) grid = tiles;
-  if (grid < 1) grid = 1;
-  return (int)grid;
+  bool ok = false;
+  if (!fwd_staging(d, n_f, &chunk, &smem, &counted)) return fwd_grid(d, n_f, n, &ok);
+  return tile_grid(d, chunk, counted, n);
+}
+// Rows of a queried workspace: fwd_grid's most over every call of up to n samples.  The grid of the
+// 128-sample tile grows with n; that of the tile of few samples does up to its last n and is above it.
+int fwd_most_rows(const tami_diagram* d, int n_f, long long n) {
+  size_t smem = 0;
+  int chunk = 0;
+  bool ok = false;
+  if (!fwd_staging(d, n_f, &chunk, &smem)) return fwd_grid(d, n_f, n, &ok);
+  const int rows = tile_grid(d, chunk, smem, n);
+  if (!coop_fits(d, n_f, &chunk, &smem)) return rows;
+  return std::max(rows, coop_grid(d, chunk, smem, std::min(n, coop_most_samples(d->device))));
 }
 
 // Momentum sampling (Sec. 5.2) appends one external momentum to the sampled ones: the calls
@@ -585,8 +606,7 @@ int tami_forward_workspace(const tami_diagram* d, int64_t n_samples, int n_f, si
   int rc = check_common(d, n_f);
   if (rc) return rc;
   if (!bytes || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
-  int grid = grid_for(d, n_f, n_samples);
-  *bytes = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
+  *bytes = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)fwd_most_rows(d, n_f, n_samples);
   return TAMI_OK;
 }
 
@@ -602,9 +622,15 @@ int tami_forward(const tami_diagram* d, const tami_lattice* lat, uint64_t seed, 
   if (!beta_ok(beta)) return TAMI_EINVAL;
   if (((uintptr_t)workspace & 255) != 0) { set_error("workspace must be 256-byte aligned"); return TAMI_EINVAL; }
   bool generic_ok = true;
-  const int grid = grid_for(d, n_f, n_samples, &generic_ok);
-  const size_t need = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
-  if (workspace_bytes < need) { set_error("workspace too small"); return TAMI_EINVAL; }
+  int grid = fwd_grid(d, n_f, n_samples, &generic_ok);
+  const size_t row = sizeof(double) * 4 * (size_t)n_f;
+  if (workspace_bytes < kHeadBytes + row * (size_t)grid) {
+    if (workspace_bytes < kHeadBytes + row * (size_t)fwd_least_rows(d, n_f, n_samples)) {
+      set_error("workspace too small");
+      return TAMI_EINVAL;
+    }
+    grid = (int)((workspace_bytes - kHeadBytes) / row);
+  }
   tami_diagram* dm = const_cast<tami_diagram*>(d);
   const int sel = jit_select(dm, kJitKindFwd, n_samples, n_f, generic_ok);
   if (sel < 0) return -sel;
@@ -645,16 +671,17 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
   if (!lat || !X || !mean || n_samples < 1) { set_error("bad argument"); return TAMI_EINVAL; }
   if (!beta_ok(beta)) return TAMI_EINVAL;
   bool generic_ok = true;
-  int grid = grid_for(d, n_f, n_samples, &generic_ok, false);
+  int grid = fwd_grid(d, n_f, n_samples, &generic_ok);
   if (!generic_ok) return TAMI_EUNSUPPORTED;   // this call runs the generic kernel only
-  const size_t need = kHeadBytes + sizeof(double) * 4 * (size_t)n_f * (size_t)grid;
+  const int least = fwd_least_rows(d, n_f, n_samples);
+  const size_t row = sizeof(double) * 4 * (size_t)n_f, need = kHeadBytes + row * (size_t)least;
   if (need > kNoAllocScratchBytes) {
     set_error("tami_forward_noalloc: needs " + std::to_string(need) + " bytes of scratch for n_f=" +
-              std::to_string(n_f) + " over " + std::to_string(grid) + " blocks, above the fixed " +
+              std::to_string(n_f) + " over " + std::to_string(least) + " blocks, above the fixed " +
               std::to_string(kNoAllocScratchBytes) + "-byte array; use tami_forward with a workspace");
     return TAMI_EINVAL;
   }
-  grid = std::min(grid_for(d, n_f, n_samples), (int)((kNoAllocScratchBytes - kHeadBytes) / (sizeof(double) * 4 * (size_t)n_f)));
+  grid = (int)std::min((size_t)grid, (kNoAllocScratchBytes - kHeadBytes) / row);
   unsigned char* base = noalloc_scratch(d->device);
   if (!base) return TAMI_ECUDA;
   cudaStream_t st = (cudaStream_t)stream;

@@ -1,4 +1,6 @@
 """What the evaluating calls accept: limits that hold at every sample count, and workspaces."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -45,3 +47,72 @@ def test_table_that_only_the_small_tile_could_hold():
         assert e.value.code == L.TAMI_EUNSUPPORTED
     m, _, p = D.forward(LAT, 7, 0, 30000, X[:242], 5.0, per_sample=True)
     assert torch.all((m - p.mean(dim=1)).abs() <= 1e-13 * p.abs().mean(dim=1))
+
+
+# ------------------------------------------------------------------------------- workspaces
+def ptr(t):
+    return ctypes.c_void_p(t.data_ptr())
+
+
+def queried(D, call, n, n_f):
+    b = ctypes.c_size_t()
+    L.check(getattr(L.lib(), f"tami_{call}_workspace")(D._h, n, n_f, ctypes.byref(b)))
+    return b.value
+
+
+def run(D, call, n, X, nbytes):
+    """The call in a workspace of nbytes; its reduced outputs."""
+    n_f, lib = len(X), L.lib()
+    ws = torch.empty((nbytes + 255) // 256 * 256, dtype=torch.uint8, device="cuda")
+    Xp = torch.view_as_real(X).contiguous()
+    g = torch.view_as_real(torch.full((n_f,), 0.5 + 0.25j, dtype=torch.complex128, device="cuda")).contiguous()
+    out = [torch.zeros((n_f, 2), dtype=torch.float64, device="cuda") for _ in range(3)] + [
+        torch.zeros(n_f, dtype=torch.float64, device="cuda"), torch.zeros(3, dtype=torch.float64, device="cuda")]
+    mean, var, dX, gX, gp = out
+    lat, st = L.Lattice(*LAT), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    head = (D._h, ctypes.byref(lat), 7, 11, n, ptr(Xp), n_f, 5.0)
+    if call == "forward":
+        L.check(lib.tami_forward(*head, ptr(mean), ptr(var), None, None, ptr(ws), nbytes, st))
+    elif call == "backward":
+        L.check(lib.tami_backward(*head, ptr(g), ptr(dX), ptr(gX), ptr(gp), None, None, None, ptr(ws), nbytes, st))
+    else:
+        L.check(lib.tami_forward_backward(*head, ptr(g), ptr(mean), ptr(var), None, ptr(dX), ptr(gX), ptr(gp), None, None,
+                                          ptr(ws), nbytes, st))
+    torch.cuda.synchronize()
+    return out
+
+
+CALLS = ["forward", "backward", "forward_backward"]
+
+
+@pytest.mark.parametrize("n_f", [5, 16, 64])
+@pytest.mark.parametrize("call", CALLS)
+def test_workspace_for_more_samples_serves_fewer(call, n_f):
+    """Around the sample counts where the small tile and the lanes that share a sample come in."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    X = torch.as_tensor(W.matsubara(5.0, n_f), device="cuda")
+    edges = [128 * sms, 256 * sms, 96 * sms, 192 * sms, 384 * sms]
+    ns = sorted({1, 33, 4000} | {e + d for e in edges for d in (-1, 0, 1)} | {100000})
+    for D in (sigma(2, 0), sigma(4, 2)):
+        sizes = [queried(D, call, n, n_f) for n in ns]
+        assert sizes == sorted(sizes)
+        for e in edges:
+            for a, b in zip(run(D, call, e, X, queried(D, call, e, n_f)), run(D, call, e, X, queried(D, call, e + 1, n_f))):
+                assert torch.equal(a, b)          # the same grid, so the same sums
+
+
+@pytest.mark.parametrize("call", CALLS)
+def test_workspace_of_one_row_per_128_samples(call):
+    """The rows that one block per 128 samples fills are enough (a workspace queried for more
+    frequencies holds no more): only the sums' grouping changes.  One row less is refused."""
+    n, n_f = 5000, 16
+    X = torch.as_tensor(W.matsubara(5.0, n_f), device="cuda")
+    D = sigma(4, 2)
+    row = 8 * {"forward": 4 * n_f, "backward": 2 * n_f + 3, "forward_backward": 6 * n_f + 3}[call]
+    least = 256 + row * -(-n // 128)
+    assert queried(D, call, n, n_f) > least
+    for a, b in zip(run(D, call, n, X, least), run(D, call, n, X, queried(D, call, n, n_f))):
+        assert torch.all((a - b).abs() <= 1e-12 * b.abs().max())
+    with pytest.raises(L.TamiError) as e:
+        run(D, call, n, X, least - 1)
+    assert e.value.code == L.TAMI_EINVAL
