@@ -619,7 +619,9 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     }
   } else {
     o("  double* Xs = smem; double* Gs = Xs + 2 * n_f; double* AXI = Gs + 2 * n_f; double* AXI2 = AXI + %d * n_f;", h.n_cden);
-    o("  double* red = AXI2 + %d * n_f;", h.n_cden);
+    // the reduction's buffer: the forward's, of 1024 threads, over the frequency constants
+    if (kind == kKindFwd) o("  double* red = smem;");
+    else o("  double* red = AXI2 + %d * n_f;", h.n_cden);
     o("  (void)AXI; (void)AXI2; (void)G; (void)ps_dX; (void)ps_grad; (void)ps_v; (void)saved;");
     o("  for (int i = tid; i < 2 * n_f; i += %d) { Xs[i] = X[i]; Gs[i] = %s; }", B, adj ? "G[i]" : "0.0");
   }
@@ -968,6 +970,7 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     return o.s;
   }
   // ---- block reduction into the generic kernel's per-block layout
+  if (kind == kKindFwd) o("  __syncthreads();");
   o("  const int nval = %s, warp = tid >> 5, lane = tid & 31;", nval);
   o("  for (int i = 0; i < nval; ++i) {");
   if (kind == kKindFused) {
@@ -1185,10 +1188,17 @@ int jit_prepare(tami_diagram* d, int kind) {
 
 // Whether an evaluating call of this kind takes the specialised kernel for n samples (compiling it if
 // so): 1 = use it, 0 = the generic kernel, or -status (the "always" mode when it cannot be built).
+// Shared memory of a specialised kernel: the frequency constants, and beside them (the forward: over
+// them) the block reduction's [warp][32] buffer.
 size_t jit_smem(const TableHeader& h, int kind, int n_f, int block) {
   if (kind == kKindEnergy) return sizeof(double) * (size_t)(2 * h.n_xk + 2 * h.n_cden) * n_f;
-  const size_t red = (size_t)block;   // the block reduction's [warp][32] buffer
-  return sizeof(double) * ((size_t)(4 + 2 * h.n_cden) * n_f + red);
+  const size_t freq = (size_t)(4 + 2 * h.n_cden) * n_f, red = (size_t)block;
+  return sizeof(double) * (kind == kKindFwd ? std::max(freq, red) : freq + red);
+}
+// The limits count the buffer of a 512-thread block beside the constants for every Monte Carlo kind.
+bool jit_fits(const TableHeader& h, int kind, int n_f, size_t optin) {
+  const size_t counted = kind == kKindEnergy ? 0 : sizeof(double) * ((size_t)(4 + 2 * h.n_cden) * n_f + 512);
+  return (kind == kKindEnergy || n_f <= kJitMaxFreq) && counted <= optin && jit_smem(h, kind, n_f, lockstep_block(h, kind)) <= optin;
 }
 
 int jit_select(tami_diagram* d, int kind, int64_t n, int n_f, bool generic_ok) {
@@ -1200,8 +1210,7 @@ int jit_select(tami_diagram* d, int kind, int64_t n, int n_f, bool generic_ok) {
   if (mode == TAMI_JIT_AUTO && !big) return 0;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, d->device);
-  const bool fits = (kind == kKindEnergy || n_f <= kJitMaxFreq) &&
-                    jit_smem(d->hdr, kind, n_f, lockstep_block(d->hdr, kind)) <= (size_t)optin;
+  const bool fits = jit_fits(d->hdr, kind, n_f, (size_t)optin);
   if (mode == TAMI_JIT_AUTO && (!fits || !jit_supported(d->hdr, kind, nullptr))) return 0;
   if (!fits) { set_error("specialised kernel: frequencies beyond its per-thread sums or shared memory"); return -TAMI_EUNSUPPORTED; }
   const int rc = jit_prepare(d, kind);
@@ -1278,7 +1287,7 @@ int jit_select_batch(tami_diagram* const* ds, int n_d, const int64_t* n, int n_f
   std::vector<int> todo;
   for (int d = 0; d < n_d; ++d) {
     std::string why;
-    const bool fits = n_f <= kJitMaxFreq && jit_smem(ds[d]->hdr, kKindFwd, n_f, lockstep_block(ds[d]->hdr, kKindFwd)) <= (size_t)optin;
+    const bool fits = jit_fits(ds[d]->hdr, kKindFwd, n_f, (size_t)optin);
     const bool ok = fits && jit_supported(ds[d]->hdr, kKindFwd, &why);
     if (mode == TAMI_JIT_AUTO && (n[d] < (int64_t(1) << 20) || !ok)) continue;
     if (!ok) {

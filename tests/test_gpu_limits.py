@@ -49,6 +49,25 @@ def test_table_that_only_the_small_tile_could_hold():
     assert torch.all((m - p.mean(dim=1)).abs() <= 1e-13 * p.abs().mean(dim=1))
 
 
+def test_many_denominators_at_many_frequencies():
+    """7 lines nu and 8 lines nu + X, 56 complex denominators: at 243 frequencies the constants of the
+    specialised forward leave less than 8 KB, and the generic kernels cannot stage the table.  The
+    call runs in every mode that compiles, as with fewer frequencies.  (Lines of one momentum have one
+    energy, so every denominator of the two groups vanishes and the values are NaN.)"""
+    if torch.cuda.get_device_properties(0).shared_memory_per_block_optin != 232448:
+        pytest.skip("stated for 232 448 bytes of shared memory per block")
+    D = T.Diagram([[1, 0]] * 7 + [[1, 1]] * 8).upload(0)
+    assert D.info()["n_cplx_dens"] == 56
+    X = torch.as_tensor(W.matsubara(5.0, 243), device="cuda")
+    T.set_jit("always")
+    few = D.forward(LAT, 7, 0, 1000, X[:100], 5.0, per_sample=True)[2]
+    for mode in ("always", "auto"):
+        T.set_jit(mode)
+        m, _, p = D.forward(LAT, 7, 0, 1000, X, 5.0, per_sample=True)
+        assert torch.equal(torch.view_as_real(p[:100]).isnan(), torch.view_as_real(few).isnan())
+        assert torch.equal(torch.view_as_real(m).isnan(), torch.view_as_real(p.mean(dim=1)).isnan())
+
+
 # ------------------------------------------------------------------------------- workspaces
 def ptr(t):
     return ctypes.c_void_p(t.data_ptr())
