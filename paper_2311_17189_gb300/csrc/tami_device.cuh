@@ -7,7 +7,6 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
-#include <vector>
 
 #include "tami_internal.h"
 #include "tami_devmath.cuh"
@@ -148,28 +147,17 @@ inline DeviceProps device_props(int dev) {
 
 // Resident blocks per SM of one of the library's kernels at `block` threads and `smem` bytes of
 // dynamic shared memory (at least 1), its shared-memory limit raised as needed.  The two runtime
-// queries take several microseconds, as long as a small launch, and every call asks for the same
-// few combinations: the answers are kept per device, kernel, block and size (a table of at most
-// kMost entries; the kernels are the library's own, so their addresses stay).
+// queries take several microseconds, as long as a small launch, so the answers are kept
+// (LaunchSizes; the kernels are the library's own, so their addresses stay).
 inline int resident_blocks(int dev, const void* kernel, int block, size_t smem) {
-  struct Known { int dev; const void* kernel; int block; size_t smem; int per_sm; };
-  constexpr size_t kMost = 256;
-  static std::mutex mu;
-  static std::vector<Known> known;
-  std::lock_guard<std::mutex> lk(mu);
-  size_t limit = 0;
-  for (const Known& k : known)
-    if (k.dev == dev && k.kernel == kernel) {
-      if (k.block == block && k.smem == smem) return k.per_sm;
-      if (k.smem > limit) limit = k.smem;
-    }
-  // the limit only grows: a smaller one set for one call would fail another thread's launch
-  if (smem > limit || limit == 0) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess) per_sm = 1;
-  if (per_sm < 1) per_sm = 1;
-  if (known.size() < kMost) known.push_back({dev, kernel, block, smem, per_sm});
-  return per_sm;
+  static LaunchSizes sizes;
+  return sizes.resident(
+      dev, kernel, block, smem,
+      [&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess; },
+      [&] {
+        int per_sm = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) == cudaSuccess ? per_sm : 1;
+      });
 }
 
 // Launches `kernel` so that its launch overlaps the end of the stream's previous kernel

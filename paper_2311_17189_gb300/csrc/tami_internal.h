@@ -2,10 +2,12 @@
 // device term table the kernels read.  Not part of the public ABI.
 #pragma once
 
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <cstdint>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <stdexcept>
 #include <string>
@@ -167,6 +169,45 @@ inline std::vector<int> phase2_program(int n_cden, int g2_const, int n_g2, const
   }
   return prog;
 }
+
+// What is known of the library's kernels on each device: the shared-memory limit that was set, and
+// the resident blocks per SM at the sizes asked for last.  A limit only grows, for the life of the
+// process (a smaller one set for one call would fail another thread's launch), and there is one per
+// kernel and device.  Sizes change with the table and n_f, so of the answers the last kMost are kept,
+// the oldest replaced.
+class LaunchSizes {
+ public:
+  static constexpr size_t kMost = 256;
+  // raise(): set the kernel's limit to smem, and whether that worked; query(): ask for its resident blocks
+  template <class Raise, class Query>
+  int resident(int dev, const void* kernel, int block, size_t smem, Raise raise, Query query) {
+    std::lock_guard<std::mutex> lk(mu_);
+    for (const Known& k : known_)
+      if (k.kernel == kernel && k.smem == smem && k.block == block && k.dev == dev) return k.per_sm;
+    Limit* limit = nullptr;
+    for (Limit& l : limits_)
+      if (l.kernel == kernel && l.dev == dev) limit = &l;
+    if (!limit) {
+      limits_.push_back({dev, kernel, 0});
+      limit = &limits_.back();
+    }
+    if ((limit->smem == 0 || smem > limit->smem) && raise()) limit->smem = smem;
+    const int per_sm = std::max(1, query());
+    const Known k{dev, kernel, block, smem, per_sm};
+    if (known_.size() < kMost) known_.push_back(k);
+    else known_[next_++ % kMost] = k;
+    return per_sm;
+  }
+  size_t answers() const { return known_.size(); }
+
+ private:
+  struct Known { int dev; const void* kernel; int block; size_t smem; int per_sm; };
+  struct Limit { int dev; const void* kernel; size_t smem; };
+  std::mutex mu_;
+  std::vector<Known> known_;
+  std::vector<Limit> limits_;
+  size_t next_ = 0;
+};
 
 }  // namespace tami
 
