@@ -288,10 +288,11 @@ int tami_forward_noalloc(const tami_diagram* d, const tami_lattice* lat, uint64_
  * for sm_103a with NVRTC (loaded at run time: libnvrtc.so.13, or the path in $TAMI_NVRTC; "none"
  * disables it) and cached with the diagram until tami_destroy.  Values agree with the generic kernels to rounding; workspaces and
  * outputs are those of the generic calls.  Part of their double products run on the integer
- * pipes, bit for bit the FP64 unit's for normal values; for tables of at most 256 pole-DAG ops the
- * per-sample products among them flush results below 2^-1022 (and subnormal operands) to zero.
- * The Monte Carlo kinds run 512-thread blocks, two per SM, whose warps meet at barriers in the
- * straight-line per-sample code.  tami_forward_noalloc always runs the generic kernel;
+ * pipes, bit for bit the FP64 unit's for normal values; in the
+ * Monte Carlo kinds of tables of at most 256 pole-DAG ops the per-sample products among them, the same
+ * ones in every kind, flush results below 2^-1022 (and subnormal operands) to zero.
+ * The Monte Carlo kinds run blocks of 512 threads, two per SM, or 1024 (the forward), whose warps meet
+ * at barriers in the straight-line per-sample code.  tami_forward_noalloc always runs the generic kernel;
  * batches take the specialised forward kernels of their large diagrams (tami_batch_plan).
  * Compiled kernels are also kept on disk, one file per compilation, in $TAMI_JIT_CACHE (default
  * $HOME/.cache/libtami_jit; "none": no disk cache): an entry records the NVRTC version, options,
@@ -430,8 +431,8 @@ int tami_selftest_sincos(const double* k, int64_t n, double* s, double* c, tami_
  * taken for normal operands with a normal result.  a, b, mul: device double [n]. */
 int tami_selftest_imul(const double* a, const double* b, int64_t n, double* mul, tami_stream_t stream);
 
-/* Diagnostic: the call-free variant of that product (imul_ftz), which large tables' specialised
- * kernels use for their per-sample products, applied elementwise: for normal operands with a
+/* Diagnostic: the call-free variant of that product (imul_ftz), which the Monte Carlo
+ * specialised kernels of tables up to 256 pole-DAG ops use for some of their per-sample products, applied elementwise: for normal operands with a
  * normal result the IEEE product, bit for bit; otherwise flush to zero — a zero or subnormal
  * operand, or a result below 2^-1022, gives a signed zero, a result above the range a signed
  * infinity, an infinite operand a signed infinity (a NaN against a zero or subnormal operand), a

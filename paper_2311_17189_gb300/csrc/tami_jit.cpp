@@ -229,6 +229,11 @@ bool keep_rr() {
 // all 17.4), larger ones, whose registers spill, none (order 5 fused 6.42 against 6.66 ms with 30 %).
 // The reverse sweep keeps its products on the FP64 unit (order 4 17.9 ms with all of them moved,
 // order 5 6.99 against 6.42 ms): there the integer product's registers cost more than its slots.
+// Values come from the same products in every Monte Carlo kind, so that their bits agree where some
+// of them are flushed: the share is the fused kind's (the forward's own, which leaves more to the
+// FP64 unit, would take 1 to 4 % less time on order 4, and the fused pass 2.7 % more with it).  Larger
+// tables and the energy input flush nothing: W1 on the FP64 unit instead of imul_ftz takes between
+// 6 % less and as much time (order 5, ten tables; order 6).
 // $TAMI_JIT_PSMUL=0 keeps every product on the FP64 unit, =all moves every one, =fwd every one of
 // the forward part.
 bool flushes(const TableHeader& h, int kind) { return kind != kKindEnergy && h.n_ops <= 256; }
@@ -507,9 +512,8 @@ bool jit_supported(const TableHeader& h, int kind, std::string* why) {
 namespace {
 
 // CUDA C++ source of the specialised kernel of one kind for one table, with the given shares of the
-// per-sample products on the integer pipes; part: where its forward part and its reverse sweep
-// begin and end.
-std::string write_source(const TableHeader& h, const unsigned char* blob, int kind, PsShare share, size_t (*part)[2]) {
+// per-sample products on the integer pipes; part: where its forward part begins and ends.
+std::string write_source(const TableHeader& h, const unsigned char* blob, int kind, PsShare share, size_t* part) {
   // The kernels are written out into more code than the instruction caches hold, so their Fermi
   // segments call one out-of-line copy of the exponential, reciprocal and selects, and their lines
   // one of the line energy (the barrier after the lines, below, has the block's warps start the
@@ -519,12 +523,16 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
   // (the energy-input kind keeps its per-row products on the FP64 unit: 1.093 -> 1.125 ms with them
   // on the integer pipes on the paper's energy-input example)
   if (kind == kKindEnergy) share = PsShare{0.0, 0.0};
-  Spread spread{share.fwd};
-  auto PM = [&](const std::string& a, const std::string& b) {
-    return spread.next() ? "imul_ftz(" + a + ", " + b + ")" : a + " * " + b;
+  // the products that form values and those that only an adjoint needs, chosen apart: every kind
+  // gives the same value products to the integer pipes
+  Spread spread{share.fwd}, adj_spread{share.fwd};
+  auto product = [&](Spread& which, const std::string& a, const std::string& b) {
+    return which.next() ? "imul_ftz(" + a + ", " + b + ")" : a + " * " + b;
   };
+  auto PM = [&](const std::string& a, const std::string& b) { return product(spread, a, b); };
+  auto AM = [&](const std::string& a, const std::string& b) { return product(adj_spread, a, b); };
   const Table t{h, blob};
-  const bool energy = kind == kKindEnergy;
+  const bool energy = kind == kKindEnergy, ftz = share.fwd > 0.0;
   const bool fwd = kind != kKindBwd, adj = kind == kKindFused || kind == kKindBwd;
   const int* repl = t.I(h.off_repl);
   const int* lm_ptr = t.I(h.off_lm_ptr);
@@ -564,6 +572,13 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
   o("#define TAMI_LINE_INLINE static __noinline__");
   o("#include \"tami_devmath.cuh\"");
   o("using namespace tami::dev;");
+  // W1 = pv RR on the FP64 unit: a plain product may be contracted into W2's sum in one kind and not in
+  // another, and the kinds' values would differ in the last bit
+  const bool factors = !ftz && !energy && h.n_rden > 0;
+  if (factors)
+    o("struct Factor { double v; __device__ operator double() const { return v; } __device__ void operator=(double x) { v = x; }\n"
+      "  __device__ void operator*=(double x) { v = v * x; } };\n"
+      "__device__ double operator*(double a, const Factor& b) { return __dmul_rn(a, b.v); }");
   if (h.n_cden > 0) {
     std::string a, k;
     for (int c = 0; c < h.n_cden; ++c) {
@@ -652,7 +667,7 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
   o("  }");
   o("  const long long n_tiles = (n + %d) / %d;", B - 1, B);
   o("  for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {");
-  part[0][0] = o.s.size();
+  if (part) part[0] = o.s.size();
   if (ls) {
     // every thread reaches every barrier: a lane past the end runs the last sample again and
     // neither adds nor writes
@@ -741,9 +756,9 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     // (g and h alike: the first derivative is symmetric in them)
     bool has_k1 = false;
     for (int v = sgm[3]; v < sgm[4]; ++v) has_k1 |= fvr[2 * v + 1] == 1;
-    const std::string d1 = (adj || has_k1)
-        ? PM("-beta", "(" + PM("sg" + std::to_string(b) + "_g", "sg" + std::to_string(b) + "_h") + ")")
-        : std::string("0.0");
+    Spread& d1_spread = has_k1 ? spread : adj_spread;
+    const std::string gh = product(d1_spread, "sg" + std::to_string(b) + "_g", "sg" + std::to_string(b) + "_h");
+    const std::string d1 = adj || has_k1 ? product(d1_spread, "-beta", "(" + gh + ")") : std::string("0.0");
     o("    double sg%d_g, sg%d_h, sg%d_d1;", b, b, b);
     o("    { const double2 gh = tami_seg_%s(x%d, beta);", bose ? "bose" : "fermi", sgm[0]);
     o("      sg%d_g = gh.x; sg%d_h = gh.y; sg%d_d1 = %s; }", b, b, b, d1.c_str());
@@ -755,7 +770,7 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     // with k = 1 values (an h value's is -d2)
     if (adj && has_k1)
       o("    const double sg%d_d2 = %s;", b,
-        PM("(" + PM("-beta", "sg" + std::to_string(b) + "_d1") + ")", "(sg" + std::to_string(b) + "_h - sg" + std::to_string(b) + "_g)").c_str());
+        AM("(" + AM("-beta", "sg" + std::to_string(b) + "_d1") + ")", "(sg" + std::to_string(b) + "_h - sg" + std::to_string(b) + "_g)").c_str());
     for (int v = sgm[3]; v < sgm[4]; ++v) {
       const bool pos = fvr[2 * v] > 0;
       const int k = fvr[2 * v + 1];
@@ -803,18 +818,19 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
       bool first = true;
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q)
         for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) {
-          if (first) o("    double RR_%d = rr%d;", gi, g1rd[2 * q]);
+          if (first && factors) o("    Factor RR_%d; RR_%d = rr%d;", gi, gi, g1rd[2 * q]);
+          else if (first) o("    double RR_%d = rr%d;", gi, g1rd[2 * q]);
           else if (spread.next()) o("    RR_%d = imul_ftz(RR_%d, rr%d);", gi, gi, g1rd[2 * q]);
           else o("    RR_%d *= rr%d;", gi, g1rd[2 * q]);
           first = false;
         }
-      // (imul_ftz: a plain product could be contracted into W2's sum, in one kind and not in another)
-      o("    double W1_%d = imul_ftz(%s, RR_%d);", gi, root_pv(gi).c_str(), gi);
+      o(ftz ? "    double W1_%d = imul_ftz(%s, RR_%d);" : "    double W1_%d = %s * RR_%d;", gi, root_pv(gi).c_str(), gi);
     } else {
       o("    double W1_%d = %s;", gi, root_pv(gi).c_str());
       for (int q = g1[4 * gi + 2]; q < g1[4 * gi + 3]; ++q)
         for (int pw = g1rd[2 * q + 1]; pw > 0; --pw) {
-          o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
+          if (ftz) o("    W1_%d = imul_ftz(W1_%d, rr%d);", gi, gi, g1rd[2 * q]);
+          else o("    W1_%d *= rr%d;", gi, g1rd[2 * q]);
         }
     }
     o(has_w2[g1_tgt[gi]] ? "    W2_%d += W1_%d;" : "    W2_%d = W1_%d;", g1_tgt[gi], gi);
@@ -830,13 +846,13 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
         if (g2cd_p[q] == 1.0 || g2cd_p[q] == -1.0)
           o("    const double pW%d = %sW2_%d;", q, g2cd_p[q] > 0 ? "" : "-", g);
         else
-          o("    const double pW%d = %s;", q, PM(lit(g2cd_p[q]), "W2_" + std::to_string(g)).c_str());
+          o("    const double pW%d = %s;", q, AM(lit(g2cd_p[q]), "W2_" + std::to_string(g)).c_str());
       }
     }
     for (int c = 0; c < h.n_cden; ++c) o("    double bb%d = 0.0;", c);
   }
   // ---- phase 2 over frequencies
-  part[0][1] = o.s.size();
+  if (part) part[1] = o.s.size();
   auto loop = [&](bool xr_zero) {
     Out whole;
     emit_phase2(whole, t, kind, xr_zero, 1.0);
@@ -850,7 +866,6 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
   if (adj) {
     if (h.g2_const) o("    Wb2_0 = s_gsum;");
     // ---- reverse sweep
-    part[1][0] = o.s.size();
     spread = Spread{share.rev};
     const bool ft = first_terms();
     for (int u = 0; u < h.n_combo; ++u) o(ft ? "    double xbar%d;" : "    double xbar%d = 0.0;", u);
@@ -962,7 +977,6 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
     o("      gmu += mub; gkx += kxb; gky += kyb;");
     o("      if (ps_grad) { ps_grad[3 * s] = mub; ps_grad[3 * s + 1] = kxb; ps_grad[3 * s + 2] = kyb; }");
     o("    }");
-    part[1][1] = o.s.size();
   }
   o("  }");
   if (energy) {   // every value is an output; nothing is reduced
@@ -1002,10 +1016,13 @@ std::string write_source(const TableHeader& h, const unsigned char* blob, int ki
 }  // namespace
 
 std::string jit_source(const TableHeader& h, const unsigned char* blob, int kind) {
-  size_t part[2][2] = {{0, 0}, {0, 0}};
-  const std::string whole = write_source(h, blob, kind, PsShare{1.0, 1.0}, part);
-  auto share = [&](int i) { return balanced_share(whole.substr(part[i][0], part[i][1] - part[i][0]), 0.0); };
-  return write_source(h, blob, kind, ps_share(PsShare{h.n_ops <= 256 ? share(0) : 0.0, 0.0}), part);
+  double share = 0.0;
+  if (flushes(h, kind)) {   // the fused kind's, for every kind
+    size_t part[2];
+    const std::string whole = write_source(h, blob, kKindFused, PsShare{1.0, 1.0}, part);
+    share = balanced_share(whole.substr(part[0], part[1] - part[0]), 0.0);
+  }
+  return write_source(h, blob, kind, ps_share(PsShare{share, 0.0}), nullptr);
 }
 
 // --------------------------------------------------------------------------- disk cache entries
