@@ -495,16 +495,28 @@ bool bwd_generic_ok(const tami_diagram* d, int n_f, bool fwd) {
 }
 
 // log2 of the lanes that share a sample: each repeats the sample's forward part and reverse sweep and
-// takes every Q-th frequency.  Launches of few samples and many frequencies are one thread's serial
-// walk long; up to 8 lanes, while every lane keeps four frequencies and six blocks per SM hold all
-// threads (order 3, 5000 samples x 200 frequencies 1605 -> 316 us with 8 lanes, 375 with 16; three
-// bubbles, 20 000 x 100, 1133 -> 403 us with 4; five bubbles, 50 000 x 40, 688 -> 524 us with 2; order
-// 4, 20 000 x 16, 399 -> 322 us; but order 5, 10 000 x 4, 303 -> 367 us: a lane with one frequency).
+// takes every Q-th frequency, which shortens the one thread's serial walk that a launch of few samples
+// and many frequencies waits for (order 3, 5000 samples x 200 frequencies 1605 -> 316 us with 8 lanes,
+// 375 with 16; three bubbles, 20 000 x 100, 1133 -> 403 us with 4).  Up to 8 lanes, each with four
+// frequencies or more, while six blocks per SM hold all threads, and a doubling only where its estimate
+// is 3 % below the time without it: the walk, in flops (half of the counted ones per sample, which
+// run on integer pipes, and one per pole-DAG step), times what the added threads cost the others.
+// That cost is a fit, of two sizes: it grows with the threads, faster for a large pole DAG, whose
+// per-thread arrays leave L1 (order 5, 788 steps), up to a half.  Over eight tables of orders 2 to 5
+// and bubbles, 8 to 128 frequencies and 100 to 58 368 samples the choice takes 0.4 % more time than
+// the best one on average, where as many lanes as the threads allow took up to 25 % more than one (order
+// 5, 10 000 samples x 8, fused: 501 us with one lane, 624 with two; 14 592 x 32: 908, 1034 with eight,
+// 851 with four; order 4, 40 000 x 8: 216 and 247).
 constexpr int kBwMostLanes = 3;                            // log2
 long long bwd_lane_samples(int dev, int lq) { return (6LL * kBlock * device_props(dev).sms) >> lq; }   // the most
 int bwd_lanes(const tami_diagram* d, int n_f, long long n) {
+  const double steps = d->hdr.n_ops, once = 0.5 * d->info.bwd_flops_per_sample + steps;
+  const double per_freq = d->info.fused_flops_per_sample_freq, crowd = 0.45 + 0.005 * steps;
+  auto walk = [&](int lq) { return once + per_freq * n_f / (1 << lq); };
   int lq = 0;
-  while (lq < kBwMostLanes && (8 << lq) <= n_f && n <= bwd_lane_samples(d->device, lq + 1)) ++lq;
+  while (lq < kBwMostLanes && (8 << lq) <= n_f && n <= bwd_lane_samples(d->device, lq + 1) &&
+         walk(lq + 1) * (1.0 + std::min(0.5, crowd * (double)n / (double)bwd_lane_samples(d->device, lq + 1))) < 0.97 * walk(lq))
+    ++lq;
   return lq;
 }
 
