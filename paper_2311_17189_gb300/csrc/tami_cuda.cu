@@ -342,16 +342,34 @@ bool coop_fits(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem) {
   return *smem <= optin;
 }
 
-// Whether a launch takes the tile of few samples, and how it stages its table.  (What a call refuses is fwd_staging's answer alone, at every n: some
-// tables fit beside this tile's smaller buffers only.)  Monte Carlo launches take it up to two 128-sample tiles per SM, where
-// those leave SMs idle and the tile's latency is the launch's: order 4, 16 frequencies, 5000 samples
-// 114 -> 53 us; order 3, 32 frequencies with per-sample values, 20 000 samples 86 -> 74 us, but
-// 65 537 samples 121 -> 148 us.  Energy input, which keeps no running sums, takes it at every size
+// Whether a Monte Carlo launch is shorter on the tile of few samples.  Up to two 128-sample tiles per SM
+// that tile's SMs would idle and its latency, a serial walk over the table, be the launch's (order 4,
+// 16 frequencies, 5000 samples 114 -> 53 us); but every 32 samples end in sums over the warp for each
+// frequency, which outweigh a small table's frequency loop.  A fit of both launches, in microseconds, at
+// 1 to 256 frequencies and 4000 to 38 912 samples: a frequency takes `here` on the small tile and
+// `there` on the large one (w: the flops per sample and frequency), and the rest, with one step of the
+// pole DAG less in the walk for every four, 12 us and 0.07 us a step less here.  Over nine tables of
+// orders 2 to 6 and bubbles the choice takes 0.04 % more than the better tile on average and 7 % at
+// worst, where the small one alone took up to 2.2 times the other's time (order 2, 38 912 samples x 64:
+// 165 us and 73; x 8: 38 and 39; order 3, x 64: 202 and 139; order 5, x 64: 364 and 513).
+bool coop_pays(const tami_diagram* d, int n_f, long long n) {
+  const int sms = device_props(d->device).sms;
+  if (n > coop_most_samples(d->device)) return false;
+  const double x = (double)n / ((double)kBlock * sms), w = d->info.flops_per_sample_freq;
+  const double crowd = n <= (long long)kCoopSamples * sms ? 0.5 : std::max(0.62 + 0.38 * x, x);   // tiles sharing an SM
+  const double here = crowd * (x <= 1.0 ? 0.88 + 0.0133 * w : 0.94 + 0.010 * w);
+  const double there = (x <= 1.0 ? 0.0345 : 0.040) * w;
+  return n_f * (here - there) <= 12.0 + 0.07 * d->hdr.n_ops;
+}
+
+// Whether a launch takes the tile of few samples, and how it stages its table.  (What a call refuses is
+// fwd_staging's answer alone, at every n: some tables fit beside this tile's smaller buffers only.)
+// Energy input, which keeps no running sums, takes it at every size
 // (order 4, 10 000 rows x 30 frequencies 156 -> 64 us; the evaluation example, 100 000 x 50, 103 -> 62
 // us; order 3, 300 000 x 100, 908 -> 755 us; two external frequencies, 250 000 x 100, 3.41 -> 3.02 ms).
 // Above kCoopMaxFreq frequencies a thread's running sums would not fit.
 bool coop_staging(const tami_diagram* d, int n_f, long long n, bool energy_in, int* ring_chunk, size_t* smem) {
-  if (!energy_in && n > coop_most_samples(d->device)) return false;
+  if (!energy_in && !coop_pays(d, n_f, n)) return false;
   return coop_fits(d, n_f, ring_chunk, smem);
 }
 

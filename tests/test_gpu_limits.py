@@ -135,3 +135,19 @@ def test_workspace_of_one_row_per_128_samples(call):
     with pytest.raises(L.TamiError) as e:
         run(D, call, n, X, least - 1)
     assert e.value.code == L.TAMI_EINVAL
+
+
+# ------------------------------------------------------------------------------- where the tiles change
+@pytest.mark.parametrize("n_f", [8, 64])
+@pytest.mark.parametrize("order,index", [(2, 0), (3, 0), (4, 2)])
+def test_samples_around_the_small_tiles_line(order, index, n_f):
+    """Either side of one and two 128-sample tiles per SM, where the choice of the tile changes with the
+    table and n_f: the same per-sample bits, and the mean of the samples."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    D = sigma(order, index)
+    X = torch.as_tensor(W.matsubara(5.0, n_f), device="cuda")
+    big = D.forward(LAT, 3, 9, 3 * 128 * sms + 5, X, 5.0, per_sample=True)[2]
+    for n in (32 * sms, 128 * sms, 128 * sms + 1, 192 * sms, 256 * sms, 256 * sms + 1):
+        m, _, p = D.forward(LAT, 3, 9, n, X, 5.0, per_sample=True)
+        assert torch.equal(p, big[:, :n]), n
+        assert torch.all((m - p.mean(dim=1)).abs() <= 1e-13 * p.abs().mean(dim=1)), n
