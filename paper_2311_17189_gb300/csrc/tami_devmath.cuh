@@ -160,7 +160,7 @@ __device__ __forceinline__ double rcp(double d) {
 // point a = j pi/512, |d| <= pi/1024, and
 //   cos phi = C - C (1 - cos d) - S sin d,   sin phi = S - S (1 - cos d) + C sin d
 // with 1 - cos d = d^2/2 - d^4/24 and sin d = d - d^3/6 + d^5/120 (W. J. Cody and W. Waite 1980,
-// reduction and series; truncation below 2e-18).  Values at 2^-61, within 6e-18 of the true ones;
+// reduction and series; truncation below 2e-18).  Values at 2^-61, a cosine within 1e-17 of the true one, a sine within 6e-18;
 // the sine within 5 pi/1024 of a multiple of pi comes from sin_near, relatively accurate down to 0.
 // 250 clocks of an SM quarter per warp for a cosine, 1200 with an FP64 Taylor series to r^20; a
 // line energy 373 against 1520, with its gradients 655 against 2580 (order-5 forward, 2^23 samples,
@@ -379,7 +379,7 @@ __device__ __forceinline__ FixedTrig trig_fixed(double k) {
   const unsigned long long cm = x2 - ((unsigned long long)__umulhi(x4, 178956971u) << 15);   // (1 - cos d) 2^79
   const unsigned int x3 = __umulhi(x2h, (unsigned int)(x >> 29));                   // d^3 2^56
   const unsigned int w = 2863311531u - __umulhi(x2h, 2185u);                        // (1/6 - d^2/120) 2^34
-  const unsigned long long sd = x - (((2ull * x3 + min(x3, 1u)) * w) >> 22);        // |sin d| 2^69, x3's middle
+  const unsigned long long sd = x - ((unsigned long long)__umulhi(x3, w) << 11);    // |sin d| 2^69
   const ulonglong2 cs = __ldg(reinterpret_cast<const ulonglong2*>(kTrigTab) + j);
   const unsigned long long sdn = sd << 2;                                           // 2^71
   const long long Ss = (long long)(mulhi_trunc(cs.y, sdn) >> 7);                    // S |sin d| 2^61
@@ -389,7 +389,8 @@ __device__ __forceinline__ FixedTrig trig_fixed(double k) {
   r.c = (q + 1u) & 2u ? -c : c;
   r.s = 0.0;
   if (NEED_SIN) {
-    const long long Cs = (long long)(mulhi_trunc(cs.x, sdn) >> 7);
+    const unsigned long long sds = x - (((2ull * x3 + min(x3, 1u)) * w) >> 22);       // sd to more bits, x3's middle
+    const long long Cs = (long long)(mulhi_trunc(cs.x, sds << 2) >> 7);
     long long v = (long long)(cs.y - (mulhi_trunc(cs.y, cm) >> 15));
     v = neg ? v - Cs : v + Cs;
     r.s = j <= 2u ? sin_near(k) : fixed_to_double<61>(((q >> 1) ^ (hi >> 31)) & 1u ? -v : v);
@@ -786,12 +787,15 @@ __device__ __forceinline__ double exp_neg(double t, double& em) {
   const bool low = y < 0x4000000000000000ull;
   y = low ? y << 1 : y;
   const int ey = 1022 - I - (low ? 1 : 0);
-  const double r = pack62(y, ey, 0u);
-  const bool big = hi >= 0x40900000u;                                                         // |t| >= 1024, NaN
+  double r = pack62(y, ey, 0u);
+  const bool big = hi >= 0x40900000u;                                                         // |t| >= 1024, NaN: ey < 1
   const bool nan = hi > 0x7FF00000u || (hi == 0x7FF00000u && lo != 0u);
-  double tail = nan ? t : 0.0;                                                                // e^t below 2^-1022
-  if ((FORM & kExpSubnormal) && ey < 1 && ey > -53 && !big)                                   // y 2^(ey - 11) of 2^-1074
-    tail = __longlong_as_double((long long)((y + (1ull << (10 - ey))) >> (11 - ey)));
+  if (!(FORM & kExpSubnormal)) {
+    r = ey < 1 ? (nan ? t : 0.0) : r;
+  } else if (ey < 1) {                                                                        // y 2^(ey - 11) of 2^-1074
+    r = nan ? t : 0.0;
+    if (ey > -53 && !big) r = __longlong_as_double((long long)((y + (1ull << (10 - ey))) >> (11 - ey)));
+  }
   if (NEED_EM) {
     // 1 - e^t: leading bit at 2^63 after the shift, exponent e1 of that bit
     const unsigned long long D1 = 0ull - (((0ull - D0) >> min(I, 63)) | 1ull);
@@ -802,7 +806,7 @@ __device__ __forceinline__ double exp_neg(double t, double& em) {
     const double d = pack62((D << c) >> 1, (k == 0 ? et : 1022) - c, 0x80000000u);
     em = big ? (nan ? t : -1.0) : (et == 0 ? t : d);
   }
-  return (big || ey < 1) ? tail : r;
+  return r;
 }
 
 // d^k/dx^k g at (g, h = 1 - g): (-beta)^k sum_i (-1)^i A(k,i) g^(i+1) h^(k-i), A = Eulerian
