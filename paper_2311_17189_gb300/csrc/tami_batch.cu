@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(kBlock) batch_kernel(const BatchParams P) {
     A.n = P.diags[d].n;
     for (int i = 0; i < kMaxFreqPerThread; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = 0.0;
     for (long long tile = item.tile0; tile < item.tile1; ++tile)
-      fwd_tile<false, false, STREAM>(Hs, T, A, tile, Xs, AXI, AXI2, xr_zero, CB, W, M, acc, R);
+      fwd_tile<false, false, STREAM, true>(Hs, T, A, tile, Xs, AXI, AXI2, xr_zero, CB, W, M, acc, R);
     block_reduce_store(M, n_f, acc, red, P.partial + (size_t)it * n_f * 4);
   }
 }

@@ -130,7 +130,12 @@ struct OpRing {
 // edge of the (shared-sub-sum) tree, v[dst] = F * (leaf ? A[ref] : v[ref]) + (first ? 0 : v[dst]),
 // over value slots; the root's sum is written by the group's last op.  Both operand loads use
 // in-range indices, the select picks one.  S: the stride of fv.  STREAM: the ops come from the ring.
-template <bool STREAM, int S = 1>
+// A node's first step is an fma onto 0: as an integer product (INT_STEPS: dag_step) it leaves the FP64
+// unit, but the chain waits longer for it (order 5, 10^6 samples x 3 frequencies: 2.75 ms, 2.23 with fmas;
+// order 4, x 21: 1.36 and 1.29 ms; order 6, x 21: 21.3 and 18.3 ms; tables of few steps 0 to 3 %).  The
+// batch kernel, whose five blocks per SM hide the wait, keeps the products (20 streams of orders 2 to
+// 5 x 32: 1.74 ms, 1.81 with fmas).
+template <bool STREAM, int S = 1, bool INT_STEPS = false>
 __device__ __forceinline__ double pole_tree(const TableView& T, OpRing& R, int op0, int op1, const double* fv) {
   double v[kMaxSlots];
   v[0] = 0.0;
@@ -141,7 +146,12 @@ __device__ __forceinline__ double pole_tree(const TableView& T, OpRing& R, int o
     const int ref = op.x >> kOpRefShift;
     const bool leaf = op.x & kOpLeaf;
     const double a = T.leafA[leaf ? ref : 0], b = v[leaf ? 0 : ref];
-    v[dst] = dag_step(fv[op.y * S], leaf ? a : b, v[dst], op.x & kOpFirst);
+    if (INT_STEPS) {
+      v[dst] = dag_step(fv[op.y * S], leaf ? a : b, v[dst], op.x & kOpFirst);
+    } else {
+      const double addend = (op.x & kOpFirst) ? 0.0 : v[dst];
+      v[dst] = fma(fv[op.y * S], leaf ? a : b, addend);
+    }
   }
   return v[dst];
 }
@@ -335,7 +345,7 @@ __device__ __forceinline__ void phase2_store(const TileArgs& A, int f, long long
 // freq_constants), CB [n_cden][kBlock], W [n_g2][kBlock].  STREAM: the pole-DAG program comes
 // through the ring R, which every thread of the block walks (a thread without a sample on zero
 // energies, its values dropped by phase 2).
-template <bool ENERGY_IN, bool SAVE, bool STREAM>
+template <bool ENERGY_IN, bool SAVE, bool STREAM, bool INT_STEPS = false>
 __device__ __forceinline__ void fwd_tile(const TableHeader& H, const TableView& T, const TileArgs& A,
                                          long long tile, const double* Xs, const double* AXI, const double* AXI2,
                                          bool xr_zero, double* CB, double* W, const FreqMap& M, double (*acc)[4],
@@ -418,7 +428,7 @@ __device__ __forceinline__ void fwd_tile(const TableHeader& H, const TableView& 
       for (int gi = 0; gi < H.n_g1; ++gi) {
         const int tg = T.g1_tgt[gi];
         if (tg != cur) { W[cur * kBlock + tid] = wacc; wacc = 0.0; cur = tg; }
-        double ft = pole_tree<STREAM>(T, R, T.g1[4 * gi], T.g1[4 * gi + 1], fv);
+        double ft = pole_tree<STREAM, 1, INT_STEPS>(T, R, T.g1[4 * gi], T.g1[4 * gi + 1], fv);
         for (int q = T.g1[4 * gi + 2]; q < T.g1[4 * gi + 3]; ++q) {
           const double r = rr[T.g1rd[2 * q]];
           for (int pw = T.g1rd[2 * q + 1]; pw > 0; --pw) ft = imul(ft, r);
