@@ -364,13 +364,9 @@ bool coop_pays(const tami_diagram* d, int n_f, long long n) {
 
 // Whether a launch takes the tile of few samples, and how it stages its table.  (What a call refuses is
 // fwd_staging's answer alone, at every n: some tables fit beside this tile's smaller buffers only.)
-// Energy input, which keeps no running sums, takes it at every size
-// (order 4, 10 000 rows x 30 frequencies 156 -> 64 us; the evaluation example, 100 000 x 50, 103 -> 62
-// us; order 3, 300 000 x 100, 908 -> 755 us; two external frequencies, 250 000 x 100, 3.41 -> 3.02 ms).
 // Above kCoopMaxFreq frequencies a thread's running sums would not fit.
-bool coop_staging(const tami_diagram* d, int n_f, long long n, bool energy_in, int* ring_chunk, size_t* smem) {
-  if (!energy_in && !coop_pays(d, n_f, n)) return false;
-  return coop_fits(d, n_f, ring_chunk, smem);
+bool coop_staging(const tami_diagram* d, int n_f, long long n, int* ring_chunk, size_t* smem) {
+  return coop_pays(d, n_f, n) && coop_fits(d, n_f, ring_chunk, smem);
 }
 
 template <bool E_IN, bool SAVE>
@@ -382,6 +378,25 @@ void (*coop_instance(const tami_diagram* d, int chunk))(const FwdParams) {
 template <bool E_IN, bool SAVE>
 int coop_blocks_per_sm(const tami_diagram* d, int chunk, size_t smem) {
   return resident_blocks(d->device, (const void*)coop_instance<E_IN, SAVE>(d, chunk), kBlock, smem);
+}
+
+// Whether energy input, which keeps no running sums, takes the tile of few samples (its shared memory
+// and the 128-sample tile's: coop_smem, tile_smem).  Up to two 128-sample tiles per SM always.  Beyond,
+// its frequency loop is the faster one and its barriers and its smaller share of an SM cost large
+// launches more.  Times over the other tile's, where the lines were drawn: small pole DAGs 300 000 rows
+// x 1 frequency 0.92 (order 2) to 1.04 (an order 4), 10^6 x 1 1.05 to 1.18, 10^6 x 25 0.71 to 0.99;
+// large ones that leave the large tile more than three blocks per SM (order 5) 50 000 x 1 0.71, 150 000
+// x 7 1.08, 300 000 x 25 1.04, 300 000 x 100 0.98; with three or fewer (order 6) 50 000 x 1 1.13, x 7
+// 0.90, 10^6 x 7 0.91; a single block per SM against two (order 6, 200 000 x 225) 1.20.
+bool coop_pays_energy(const tami_diagram* d, int n_f, long long n, size_t coop_smem, size_t tile_smem) {
+  const DeviceProps dp = device_props(d->device);
+  const long long full = (long long)kBlock * dp.sms;
+  auto blocks = [&](size_t smem) { return (dp.smem_optin + 1024) / (smem + 1024); };   // that share an SM's memory
+  if (n <= 2 * full) return true;
+  if (blocks(coop_smem) < 2 && blocks(tile_smem) > 1) return false;
+  if (d->hdr.n_ops <= 256) return n_f >= 16 || n <= (16 + 2 * n_f) * full;
+  if (blocks(tile_smem) <= 3) return n_f >= 4;
+  return n_f >= 64 || n <= 6 * full;
 }
 
 template <bool E_IN, bool SAVE>
@@ -403,8 +418,9 @@ int launch_fwd(const tami_diagram* d, FwdParams& P, cudaStream_t stream, int max
   size_t smem = 0, coop_smem = 0;
   int chunk = 0, coop_chunk = 0;
   if (!fwd_staging(d, P.n_f, &chunk, &smem)) return TAMI_EUNSUPPORTED;
-  if (coop_staging(d, P.n_f, P.n, E_IN, &coop_chunk, &coop_smem))
-    return launch_coop<E_IN, SAVE>(d, P, coop_chunk, coop_smem, stream, max_blocks, launched);
+  const bool coop = E_IN ? coop_fits(d, P.n_f, &coop_chunk, &coop_smem) && coop_pays_energy(d, P.n_f, P.n, coop_smem, smem)
+                         : coop_staging(d, P.n_f, P.n, &coop_chunk, &coop_smem);
+  if (coop) return launch_coop<E_IN, SAVE>(d, P, coop_chunk, coop_smem, stream, max_blocks, launched);
   P.ring_chunk = chunk;
   DeviceProps dp = device_props(d->device);
   const int per_sm = chunk ? fwd_blocks_per_sm<E_IN, SAVE, true>(d->device, smem) : fwd_blocks_per_sm<E_IN, SAVE, false>(d->device, smem);
@@ -441,7 +457,7 @@ int fwd_grid(const tami_diagram* d, int n_f, long long n, bool* generic_ok) {
   size_t coop_smem = 0;
   *generic_ok = fwd_staging(d, n_f, &chunk, &smem);
   if (!*generic_ok) return (int)std::max(1LL, std::min((n + kBlock - 1) / kBlock, 4LL * device_props(d->device).sms));
-  if (coop_staging(d, n_f, n, false, &coop_chunk, &coop_smem)) return coop_grid(d, coop_chunk, coop_smem, n);
+  if (coop_staging(d, n_f, n, &coop_chunk, &coop_smem)) return coop_grid(d, coop_chunk, coop_smem, n);
   return tile_grid(d, chunk, smem, n);
 }
 // Rows that a call asks of its workspace: the 128-sample tile's blocks, with the shared memory that the
@@ -461,9 +477,11 @@ int fwd_most_rows(const tami_diagram* d, int n_f, long long n) {
   int chunk = 0;
   bool ok = false;
   if (!fwd_staging(d, n_f, &chunk, &smem)) return fwd_grid(d, n_f, n, &ok);
-  const int rows = tile_grid(d, chunk, smem, n);
-  if (!coop_fits(d, n_f, &chunk, &smem)) return rows;
-  return std::max(rows, coop_grid(d, chunk, smem, std::min(n, coop_most_samples(d->device))));
+  int coop_chunk = 0;
+  size_t coop_smem = 0;
+  int rows = 0;
+  if (coop_fits(d, n_f, &coop_chunk, &coop_smem)) rows = coop_grid(d, coop_chunk, coop_smem, std::min(n, coop_most_samples(d->device)));
+  return rows >= (n + kBlock - 1) / kBlock ? rows : std::max(rows, tile_grid(d, chunk, smem, n));
 }
 
 // Momentum sampling (Sec. 5.2) appends one external momentum to the sampled ones: the calls

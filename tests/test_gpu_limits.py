@@ -151,3 +151,21 @@ def test_samples_around_the_small_tiles_line(order, index, n_f):
         m, _, p = D.forward(LAT, 3, 9, n, X, 5.0, per_sample=True)
         assert torch.equal(p, big[:, :n]), n
         assert torch.all((m - p.mean(dim=1)).abs() <= 1e-13 * p.abs().mean(dim=1)), n
+
+
+@pytest.mark.parametrize("order,index", [(2, 0), (5, 12)])
+def test_rows_around_the_small_tiles_line(order, index):
+    """Energy input: either side of the rows at which the tile changes, for a small and a large pole DAG,
+    with few and many frequencies: the same bits as 257 frequencies, which only the large tile takes."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    D = sigma(order, index)
+    assert (D.info()["n_dag_ops"] > 256) == (order == 5)
+    X = torch.as_tensor(W.matsubara(2.0, 257), device="cuda")
+    E = torch.as_tensor(W.random_energies(18 * 128 * sms + 1, D.n_lines, a=4.0, seed=9), device="cuda")
+    for rows in (256 * sms, 256 * sms + 1, 768 * sms, 768 * sms + 1, 18 * 128 * sms, 18 * 128 * sms + 1):
+        e = E[:rows].contiguous()
+        few = D.eval_energies(e, X[:1], 2.0)
+        for n_f in (15, 16, 65):
+            assert torch.equal(D.eval_energies(e, X[:n_f], 2.0)[:1], few), (rows, n_f)
+        tail = e[-33:].contiguous()
+        assert torch.equal(D.eval_energies(tail, X, 2.0)[:1], few[:, -33:]), rows
