@@ -411,14 +411,15 @@ int tami_set_table_staging(int mode, int chunk_ops);
  * take the value at planning time; the other calls at each launch.  Process-wide. */
 int tami_debug_set_wait_limit(int64_t first_stage_spins);
 
-/* Diagnostic: the kernels' exponential for t <= 0 (table-driven, in 64-bit fixed point), applied
+/* Diagnostic: the kernels' exponential for t <= 0 (table-driven, in 64-bit fixed point, subnormal
+ * values rounded; the specialised kernels that flush subnormal products give 0 there), applied
  * elementwise: y = e^t, em = e^t - 1, and y_plain = e^t from the variant that does not form
  * e^t - 1 (the kernels use it where only e^t is needed; it must equal y bit for bit).
  * t, y, em, y_plain: device double [n]; y_plain may be NULL.  Used by the tests to check them
  * against CUDA's exp/expm1. */
 int tami_selftest_exp(const double* t, int64_t n, double* y, double* em, double* y_plain, tami_stream_t stream);
 
-/* Diagnostic: the kernels' cos and sin (Cody-Waite reduction by pi and Taylor series, the
+/* Diagnostic: the kernels' cos and sin (64-bit fixed-point reduction, a table and short series; the
  * dispersion of Sec. 5.2's lattice samples; the paper leaves eps(k) to the user) applied
  * elementwise: s = sin k, c = cos k.  k, s, c: device double [n].  c holds NaN where the
  * cosine-only path that the energies use differs from the sin/cos path in any bit.  Used by the

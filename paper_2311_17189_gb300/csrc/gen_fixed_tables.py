@@ -1,10 +1,10 @@
-"""Writes the fixed-point tables of the kernels' exponential and cos/sin (csrc/tami_fixed_tables.cuh)
-from 60-digit values:
+"""Writes the fixed-point tables of the kernels' exponential and cos/sin, which stand in
+csrc/tami_devmath.cuh (kExpTab, kTrigTab), from 60-digit values:
 
   kExpTab[j]  = round((1 - 2^(-j/1024)) 2^64), j = 0..1023
   kTrigTab[j] = (round(cos(j pi/512) 2^61), round(sin(j pi/512) 2^61)), j = 0..256
 
-    python gen_fixed_tables.py > tami_fixed_tables.cuh
+    python gen_fixed_tables.py          # prints both tables as they stand there
 """
 import mpmath as mp
 

@@ -1,5 +1,5 @@
 // Device arithmetic of the libtami kernels: the counter-based momentum sampler, the lattice
-// dispersion with its Cody-Waite cos/sin, the table-driven exponential, the reciprocal and the
+// dispersion with its fixed-point cos/sin, the table-driven exponential, the reciprocal and the
 // Fermi/Bose values and derivatives of one table segment.  Self-contained (no host headers, plain
 // integer types), so that the same text also serves the kernels the library generates and
 // compiles at run time for one diagram's table (tami_jit.cpp).  Internal to the library.
@@ -139,11 +139,11 @@ __device__ __forceinline__ double imul_ftz(double a, double b) {
 }
 
 
-// 1/d, within 0.501 ulp, in integer arithmetic (recip_sig): 63 clocks of an SM quarter per warp on
+// 1/d, within 0.502 ulp, in integer arithmetic (recip_sig): 60 clocks of an SM quarter per warp on
 // the integer pipes, 215 on the FP64 unit for the hardware's FP64 estimate and a third-order Newton
-// step (order 3 on the real axis, 2^21 samples x 256 frequencies: 45.4 -> 39.9 ms).  A zero, subnormal or infinite d and a
-// NaN give a NaN (as the Newton step on the hardware's FP64 estimate did); |d| >= 2^1022, whose
-// reciprocal is subnormal, a signed zero.
+// step (order 3 on the real axis, 2^21 samples x 256 frequencies: 45.4 -> 39.9 ms).  A zero, subnormal
+// or infinite d and a NaN give a NaN (as the Newton step on the hardware's FP64 estimate did); |d| >=
+// 2^1022, whose reciprocal is 2^-1022 or subnormal, a signed zero.
 __device__ __forceinline__ double rcp(double d) {
   const unsigned int hi = (unsigned int)__double2hiint(d);
   const int ed = (int)(hi >> 20) & 0x7FF;
@@ -160,12 +160,12 @@ __device__ __forceinline__ double rcp(double d) {
 // point a = j pi/512, |d| <= pi/1024, and
 //   cos phi = C - C (1 - cos d) - S sin d,   sin phi = S - S (1 - cos d) + C sin d
 // with 1 - cos d = d^2/2 - d^4/24 and sin d = d - d^3/6 + d^5/120 (W. J. Cody and W. Waite 1980,
-// reduction and series; truncation below 2e-18).  Values at 2^-61, a cosine within 1e-17 of the true one, a sine within 6e-18;
-// the sine within 5 pi/1024 of a multiple of pi comes from sin_near, relatively accurate down to 0.
-// 250 clocks of an SM quarter per warp for a cosine, 1200 with an FP64 Taylor series to r^20; a
-// line energy 373 against 1520, with its gradients 655 against 2580 (order-5 forward, 2^23 samples,
-// one frequency: 9.6 -> 5.6 ms; order-4 forward + adjoint, 2^24 samples x 16 frequencies: 78.6 ->
-// 71.9 ms).
+// reduction and series; truncation below 2e-18).  Values at 2^-61, a cosine within 1e-17 of the true
+// one, a sine within 6e-18; the sine within 5 pi/1024 of a multiple of pi comes from sin_near,
+// relatively accurate down to 0.  245 clocks of an SM quarter per warp for a cosine, 1200 with an FP64
+// Taylor series to r^20; a line energy 355 against 1520, with its gradients 690 against 2580 (order-5
+// forward, 2^23 samples, one frequency: 9.6 -> 5.6 ms; order-4 forward + adjoint, 2^24 samples x 16
+// frequencies: 78.6 -> 71.9 ms).
 __device__ const __align__(16) unsigned long long kTrigTab[514] = {
   0x2000000000000000ull, 0x0000000000000000ull, 0x1fffd8858e8a924dull, 0x003243e1fcce00e2ull,
   0x1fff62169b92db57ull, 0x00648747f37b1e12ull, 0x1ffe9cb44b51a12bull, 0x0096c9b5df1877eaull,
@@ -303,7 +303,8 @@ __device__ const __align__(16) unsigned long long kTrigTab[514] = {
 // double below 32 is never closer than 1.2e-16 to a multiple of pi); then
 // sin r = r (1 - r^2/6 + r^4/120 - r^6/5040).  One argument in a hundred comes here, a warp in four for
 // one of its lanes: out of line, and in integers, as FP64 instructions would take as long as the whole
-// fixed-point sine.
+// fixed-point sine.  (Five bubbles, fused, 2^22 samples x 16 frequencies: 9.57 ms without it, 9.80 with;
+// order 4 0.3 % more.)
 static __device__ __noinline__ double sin_near(double k) {
   const unsigned int hi = (unsigned int)__double2hiint(k);
   const int ek = (int)(hi >> 20) & 0x7FF;
@@ -492,8 +493,8 @@ __device__ TAMI_LINE_INLINE double line_energy_grad(double kx, double ky, double
 // V_j = 1 - 2^(-j/1024) from the table at 2^64, p = 1 - e^-z = z (1 - s), s = z/2 - z^2/6 + z^3/24
 // - z^4/120 (truncation below 2^-58 relative).  z is formed at 2^-72 modulo 2^-8, so its bits below
 // the integer part of |t| are exact, with a 94-bit ln2/1024; |t| < ln2/1024 takes 1 - e^t = |t| (1 - s)
-// on t's own significand, so the result is relatively exact down to t = 0.  190 clocks of an SM
-// quarter per warp for e^t, 250 with e^t - 1; an FP64 polynomial after a 256-entry table took 859
+// on t's own significand, so the result is relatively exact down to t = 0.  180 clocks of an SM
+// quarter per warp for e^t, 235 with e^t - 1; an FP64 polynomial after a 256-entry table took 859
 // and 1102 (order-5 forward, 2^23 samples, one frequency: 13.3 -> 9.6 ms).  Within 0.51 ulp, e^t - 1
 // within 0.75; e^t below 2^-1022 is rounded to a subnormal value with kExpSubnormal, else 0 (for code
 // whose products flush those anyway).
