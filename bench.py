@@ -57,8 +57,8 @@ METRIC = "order-4 Sigma evals/s (samples x terms x frequencies, FP64), forward +
 # caches the compilation (whose options are fixed in the library) -- must hash to the captured
 # one, else the bench reports traffic as null.
 TRAFFIC = {"kernel": "tami_jit_fused (the diagram's specialised fused forward + adjoint)",
-           "bytes_per_sample": (4.330491e9 + 5.248207e9) / 4194304,
-           "kernel_sha256": "dd08037582d26ff2c4f542e9334d273bbe3d864a879487cb1fd69db5f741048d",
+           "bytes_per_sample": (4.400303e9 + 5.368045e9) / 4194304,
+           "kernel_sha256": "4007f6af17312a9e2e85c0bbb4a71680d924e40d81ff89f0420ed58bfb716b45",
            "profile": "profiles/jit_kernels_order4_sigma.md"}
 
 
