@@ -347,19 +347,19 @@ bool coop_fits(const tami_diagram* d, int n_f, int* ring_chunk, size_t* smem) {
 // 16 frequencies, 5000 samples 114 -> 53 us); but every 32 samples end in sums over the warp for each
 // frequency, which outweigh a small table's frequency loop.  A fit of both launches, in microseconds, at
 // 1 to 256 frequencies and 4000 to 38 912 samples: a frequency takes `here` on the small tile and
-// `there` on the large one (w: the flops per sample and frequency), and the rest, with one step of the
-// pole DAG less in the walk for every four, 12 us and 0.07 us a step less here.  Over nine tables of
-// orders 2 to 6 and bubbles the choice takes 0.04 % more than the better tile on average and 7 % at
-// worst, where the small one alone took up to 2.2 times the other's time (order 2, 38 912 samples x 64:
-// 165 us and 73; x 8: 38 and 39; order 3, x 64: 202 and 139; order 5, x 64: 364 and 513).
+// `there` on the large one (w: the flops per sample and frequency), and the rest, a walk shared by four
+// warps, 8 us and 0.03 us a pole-DAG step less here.  Over nine tables of orders 2 to 6 and bubbles the
+// choice takes 0.08 % more than the better tile on average and 7 % at worst, where the small one alone
+// took up to 2.2 times the other's time (order 2, 38 912 samples x 64: 164 us and 73; x 8: 37 and 38;
+// order 3, x 64: 201 and 136; order 5, x 64: 334 and 462).
 bool coop_pays(const tami_diagram* d, int n_f, long long n) {
   const int sms = device_props(d->device).sms;
   if (n > coop_most_samples(d->device)) return false;
   const double x = (double)n / ((double)kBlock * sms), w = d->info.flops_per_sample_freq;
-  const double crowd = n <= (long long)kCoopSamples * sms ? 0.5 : std::max(0.62 + 0.38 * x, x);   // tiles sharing an SM
-  const double here = crowd * (x <= 1.0 ? 0.88 + 0.0133 * w : 0.94 + 0.010 * w);
-  const double there = (x <= 1.0 ? 0.0345 : 0.040) * w;
-  return n_f * (here - there) <= 12.0 + 0.07 * d->hdr.n_ops;
+  const double crowd = n <= (long long)kCoopSamples * sms ? 0.5 : std::max(0.55 + 0.45 * x, x);   // tiles sharing an SM
+  const double here = crowd * (x <= 1.0 ? 0.88 + 0.0133 * w : 0.90 + 0.009 * w);
+  const double there = (x <= 1.0 ? 0.033 : 0.038) * w;
+  return n_f * (here - there) <= 8.0 + 0.03 * d->hdr.n_ops;
 }
 
 // Whether a launch takes the tile of few samples, and how it stages its table.  (What a call refuses is
