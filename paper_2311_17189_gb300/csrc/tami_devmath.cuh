@@ -161,11 +161,11 @@ __device__ __forceinline__ double rcp(double d) {
 //   cos phi = C - C (1 - cos d) - S sin d,   sin phi = S - S (1 - cos d) + C sin d
 // with 1 - cos d = d^2/2 - d^4/24 and sin d = d - d^3/6 + d^5/120 (W. J. Cody and W. Waite 1980,
 // reduction and series; truncation below 2e-18).  Values at 2^-61, a cosine within 1e-17 of the true
-// one, a sine within 6e-18; the sine within 5 pi/1024 of a multiple of pi comes from sin_near,
-// relatively accurate down to 0.  245 clocks of an SM quarter per warp for a cosine, 1200 with an FP64
-// Taylor series to r^20; a line energy 355 against 1520, with its gradients 690 against 2580 (order-5
-// forward, 2^23 samples, one frequency: 9.6 -> 5.6 ms; order-4 forward + adjoint, 2^24 samples x 16
-// frequencies: 78.6 -> 71.9 ms).
+// one, a sine within 6e-18 beside the last rounding (3.2 ulp at most); the sine within 3 pi/1024 of a
+// multiple of pi comes from sin_near, relatively accurate down to 0.  245 clocks of an SM quarter per
+// warp for a cosine, 1200 with an FP64 Taylor series to r^20; a line energy 355 against 1520, with its
+// gradients 690 against 2580 (order-5 forward, 2^23 samples, one frequency: 9.6 -> 5.6 ms; order-4
+// forward + adjoint, 2^24 samples x 16 frequencies: 78.6 -> 71.9 ms).
 __device__ const __align__(16) unsigned long long kTrigTab[514] = {
   0x2000000000000000ull, 0x0000000000000000ull, 0x1fffd8858e8a924dull, 0x003243e1fcce00e2ull,
   0x1fff62169b92db57ull, 0x00648747f37b1e12ull, 0x1ffe9cb44b51a12bull, 0x0096c9b5df1877eaull,
@@ -297,55 +297,23 @@ __device__ const __align__(16) unsigned long long kTrigTab[514] = {
   0x00648747f37b1e12ull, 0x1fff62169b92db57ull, 0x003243e1fcce00e2ull, 0x1fffd8858e8a924dull,
   0x0000000000000000ull, 0x2000000000000000ull};
 
-// sin k next to a multiple of pi (|k - n pi| < 2^-6, |k| < 32), within 0.52 ulp, where a fixed-point
-// value keeps no relative accuracy.  r = |k - n pi| is put on 64 significant bits: k's own significand
-// for n = 0, else |k| in turns, |k| 2^58 times 2^134/(2 pi), with 64 bits more than trig_fixed's (a
-// double below 32 is never closer than 1.2e-16 to a multiple of pi); then
-// sin r = r (1 - r^2/6 + r^4/120 - r^6/5040).  One argument in a hundred comes here, a warp in four for
-// one of its lanes: out of line, and in integers, as FP64 instructions would take as long as the whole
-// fixed-point sine.  (Five bubbles, fused, 2^22 samples x 16 frequencies: 9.57 ms without it, 9.80 with;
-// order 4 0.3 % more.)
-static __device__ __noinline__ double sin_near(double k) {
-  const unsigned int hi = (unsigned int)__double2hiint(k);
-  const int ek = (int)(hi >> 20) & 0x7FF;
-  if (ek < 990) return k;                                                            // |k| < 2^-33
-  unsigned int sign = hi & 0x80000000u;
-  unsigned long long m = (((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | (unsigned int)__double2loint(k)) << 11;
-  int e = ek - 1023;                                                                 // |k| = m 2^(e - 63)
-  if (e >= 0) {
-    const unsigned long long K = m >> (5 - e);                                       // |k| 2^58
-    const unsigned int kl = (unsigned int)K, kh = (unsigned int)(K >> 32);
-    const unsigned long long t0 = (unsigned long long)kl * 0xE441529Fu;
-    const unsigned long long t1 = (unsigned long long)kh * 0xE441529Fu + (t0 >> 32);
-    const unsigned long long t2 = (unsigned long long)kl * 0x2F9836E4u + (unsigned int)t1;
-    const unsigned long long low = mulhi_trunc(K, 0x613ABE8FA9A6EE06ull) << 1;
-    unsigned long long tl = ((t2 << 32) | (unsigned int)t0) + low;
-    unsigned long long th = K * 10ull + (unsigned long long)kh * 0x2F9836E4u + (t1 >> 32) + (t2 >> 32) + (tl < low ? 1u : 0u);
-    const bool odd = (long long)th < 0;                                              // half turns, |k| = (odd + (th, tl) 2^-128) pi
-    th = (th << 1) | (tl >> 63);
-    tl <<= 1;
-    const bool under = (long long)th < 0;                                            // from the next multiple down
-    if (under) {
-      th = ~th + (tl == 0ull ? 1u : 0u);
-      tl = 0ull - tl;
-    }
-    sign ^= odd ? 0x80000000u : 0u;   // (-1)^n and r's sign: n is odd + 1 where r is below 0, and the two cancel
-    const int z = min(max(__clzll((long long)th), 1), 63);
-    m = mulhi_trunc(((th << z) | (tl >> (64 - z))) >> 1, 0x6487ED5110B4611Aull) << 2;   // times pi 2^-2
-    e = 1 - z;
-    if (!(m >> 63)) { m <<= 1; --e; }
-  }
-  const unsigned long long rf = m >> min(-5 - e, 63);                                // r 2^68
-  const unsigned long long r2 = mulhi_trunc(rf, rf);                                 // r^2 2^72
-  const unsigned int r2h = (unsigned int)(r2 >> 28);                                 // r^2 2^44
-  const unsigned int q = __umulhi(r2h, 2290649225u - __umulhi(r2h, 13315u));         // (r^2/120 - r^4/5040) 2^50
-  const unsigned long long c = mulhi_trunc(r2, 0x2AAAAAAAAAAAAAABull - ((unsigned long long)q << 14));   // 1 - sin(r)/r, 2^72
-  m -= mulhi_trunc(m >> 1, c) >> 7;
-  if (!(m >> 63)) { m <<= 1; --e; }
-  return pack62(m >> 1, e + 1023, sign);
+// sin k next to a multiple of pi (|k - n pi| < 3 pi/1024, |k| < 32), where a fixed-point value keeps no
+// relative accuracy, on the FP64 unit: r = k - n pi (n the integer nearest to k/pi, from one fma against
+// 1.5 2^52; n times the first part of pi taken off exactly, the second with one rounding; a double below
+// 32 is never closer than 1.2e-16 to a multiple of pi), r (1 - r^2/6 + r^4/120 - r^6/5040) and the sign
+// (-1)^n: one rounding of r (none for n = 0) and one of the sum.  One argument in 170 comes here, a warp
+// in six for one of its lanes, so that the size of the code counts: a reduction in 64-bit integers,
+// called out of line within 5 pi/1024 (0.51 ulp), slowed the generic kernels by its instruction fetches
+// (five bubbles, fused, 1.5 10^6 samples x 2 frequencies: 2.00 ms with fixed-point sines throughout,
+// 2.44 with it, 2.07 with this; generated kernel, 2^22 x 16: 9.58, 9.81, 9.72 ms).
+__device__ __forceinline__ double sin_near(double k) {
+  const double nd = fma(k, 0x1.45f306dc9c883p-2, 0x1.8p52), n = nd - 0x1.8p52;
+  const double r = fma(-n, 0x1.1a62633145c07p-53, fma(-n, 0x1.921fb54442d18p+1, k)), z = r * r;
+  const double v = fma(r * z, fma(z, fma(z, -0x1.a01a01a01a01ap-13, 0x1.1111111111111p-7), -0x1.5555555555555p-3), r);
+  return __hiloint2double((int)((unsigned int)__double2hiint(v) ^ ((unsigned int)__double2loint(nd) << 31)), __double2loint(v));
 }
 
-struct FixedTrig { long long c; double s; };   // cos times 2^61, sin
+struct FixedTrig { long long c, s; bool near; };   // cos and sin times 2^61; near: the sine is sin_near's
 
 // v 2^-S rounded to the nearest double
 template <int S>
@@ -388,13 +356,14 @@ __device__ __forceinline__ FixedTrig trig_fixed(double k) {
   c = neg ? c + Ss : c - Ss;
   FixedTrig r;
   r.c = (q + 1u) & 2u ? -c : c;
-  r.s = 0.0;
+  r.s = 0;
+  r.near = NEED_SIN && j <= 1u;
   if (NEED_SIN) {
     const unsigned long long sds = x - (((2ull * x3 + min(x3, 1u)) * w) >> 22);       // sd to more bits, x3's middle
     const long long Cs = (long long)(mulhi_trunc(cs.x, sds << 2) >> 7);
     long long v = (long long)(cs.y - (mulhi_trunc(cs.y, cm) >> 15));
     v = neg ? v - Cs : v + Cs;
-    r.s = j <= 2u ? sin_near(k) : fixed_to_double<61>(((q >> 1) ^ (hi >> 31)) & 1u ? -v : v);
+    r.s = ((q >> 1) ^ (hi >> 31)) & 1u ? -v : v;
   }
   return r;
 }
@@ -413,14 +382,21 @@ __device__ __forceinline__ double trig_reduce(double k, bool& odd) {
   return good ? r : fmod(k, 0x1.921fb54442d18p+2);
 }
 
+__device__ __forceinline__ double trig_sin(double k, const FixedTrig& t) {
+  return t.near ? sin_near(k) : fixed_to_double<61>(t.s);
+}
+
+struct AnyTrig { long long c; double s; };   // cos times 2^61, sin
 template <bool NEED_SIN>
-__device__ __forceinline__ FixedTrig trig_any(double k, bool& finite) {
+__device__ __forceinline__ AnyTrig trig_any(double k, bool& finite) {
   bool odd = false;
   const double r = trig_far(k) ? trig_reduce(k, odd) : k;
-  FixedTrig t = trig_fixed<NEED_SIN>(r);
-  if (odd) { t.c = -t.c; t.s = -t.s; }
+  const FixedTrig t = trig_fixed<NEED_SIN>(r);
+  AnyTrig a = {t.c, 0.0};
+  if (NEED_SIN) a.s = trig_sin(r, t);
+  if (odd) { a.c = -a.c; a.s = -a.s; }
   finite = r == r;
-  return t;
+  return a;
 }
 
 __device__ __forceinline__ double cw_cos(double k) {
@@ -431,7 +407,7 @@ __device__ __forceinline__ double cw_cos(double k) {
 
 __device__ __forceinline__ void cw_sincos(double k, double& s_out, double& c_out) {
   bool finite;
-  const FixedTrig t = trig_any<true>(k, finite);
+  const AnyTrig t = trig_any<true>(k, finite);
   s_out = finite ? t.s : k - k;
   c_out = finite ? fixed_to_double<61>(t.c) : k - k;
 }
@@ -446,27 +422,19 @@ __device__ __forceinline__ double line_energy_of(long long cx, long long cy, dou
   return fma(4.0 * tp, prod, fma(2.0 * t, sum, mu));
 }
 
-template <bool GRAD>
-__device__ __forceinline__ double line_energy_from(const FixedTrig& x, const FixedTrig& y, double t, double tp, double mu,
-                                                   double& gx, double& gy) {
-  if (GRAD) {
-    gx = fma(4.0 * tp, fixed_to_double<61>(y.c), 2.0 * t) * x.s;
-    gy = fma(4.0 * tp, fixed_to_double<61>(x.c), 2.0 * t) * y.s;
-  }
-  return line_energy_of(x.c, y.c, t, tp, mu);
-}
-
 // Momenta of 32 and above (a large k_ext): out of line, so that the common path carries no FP64
 // reduction.  A momentum that is not finite gives a NaN.
 template <bool GRAD>
 static __device__ __noinline__ double line_energy_far(double kx, double ky, double t, double tp, double mu, double& gx,
                                                       double& gy) {
   bool fx, fy;
-  const FixedTrig x = trig_any<GRAD>(kx, fx), y = trig_any<GRAD>(ky, fy);
-  const double E = line_energy_from<GRAD>(x, y, t, tp, mu, gx, gy);
+  const AnyTrig x = trig_any<GRAD>(kx, fx), y = trig_any<GRAD>(ky, fy);
   const double bad = fx && fy ? 0.0 : (kx - kx) + (ky - ky);          // 0, or a NaN
-  if (GRAD) { gx += bad; gy += bad; }
-  return E + bad;
+  if (GRAD) {
+    gx = fma(4.0 * tp, fixed_to_double<61>(y.c), 2.0 * t) * x.s + bad;
+    gy = fma(4.0 * tp, fixed_to_double<61>(x.c), 2.0 * t) * y.s + bad;
+  }
+  return line_energy_of(x.c, y.c, t, tp, mu) + bad;
 }
 
 #ifndef TAMI_LINE_INLINE   // the generated kernels call one out-of-line copy
@@ -475,7 +443,7 @@ static __device__ __noinline__ double line_energy_far(double kx, double ky, doub
 __device__ TAMI_LINE_INLINE double line_energy(double kx, double ky, double t, double tp, double mu) {
   double gx, gy;
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<false>(kx, ky, t, tp, mu, gx, gy);
-  return line_energy_from<false>(trig_fixed<false>(kx), trig_fixed<false>(ky), t, tp, mu, gx, gy);
+  return line_energy_of(trig_fixed<false>(kx).c, trig_fixed<false>(ky).c, t, tp, mu);
 }
 
 // Energy of a line that carries k_ext, with the factors G = (2t + 4t' cos K_perp) sin K of
@@ -483,7 +451,10 @@ __device__ TAMI_LINE_INLINE double line_energy(double kx, double ky, double t, d
 __device__ TAMI_LINE_INLINE double line_energy_grad(double kx, double ky, double t, double tp, double mu, double& gx,
                                                    double& gy) {
   if (trig_far(kx) || trig_far(ky)) return line_energy_far<true>(kx, ky, t, tp, mu, gx, gy);
-  return line_energy_from<true>(trig_fixed<true>(kx), trig_fixed<true>(ky), t, tp, mu, gx, gy);
+  const FixedTrig x = trig_fixed<true>(kx), y = trig_fixed<true>(ky);
+  gx = fma(4.0 * tp, fixed_to_double<61>(y.c), 2.0 * t) * trig_sin(kx, x);
+  gy = fma(4.0 * tp, fixed_to_double<61>(x.c), 2.0 * t) * trig_sin(ky, y);
+  return line_energy_of(x.c, y.c, t, tp, mu);
 }
 
 // e^t and e^t - 1 for t <= 0 in fixed point, after P. T. P. Tang, "Table-driven implementation of the

@@ -4,13 +4,15 @@
 #include "fixed_math_cases.cpp"
 #undef main
 
-// 6e-18 is trig_fixed's stated bound; sin_near rounds 60 significant bits once
+// 6e-18 is trig_fixed's stated bound.  sin_near, within 3 pi/1024, rounds the distance from the zero (half
+// an ulp of it, one of a sine in the binade below) and the sum (half an ulp); its series and the third
+// part of pi add less than 0.02.
 static void one(double k, double extra_ulp) {
   double s, c;
   cw_sincos(k, s, c);
   const L ref = std::sin((L)k), err = std::fabs((L)s - ref), u = ulp((double)ref);
   const L from_zero = std::fabs((L)k - (L)M_PIl * std::round((L)k / M_PIl));
-  const L bound = from_zero < 0.0153L ? (0.52L + extra_ulp) * u : (0.5L + extra_ulp) * u + 6e-18L;
+  const L bound = from_zero < 0.0092L ? (1.52L + extra_ulp) * u : (0.5L + extra_ulp) * u + 6e-18L;
   check(err <= bound, "sin near a zero", k, s);
   check(std::fabs((double)((L)c - std::cos((L)k))) <= 1.2e-16 * (1 + extra_ulp), "cos near a zero of sin", k, c);
 }
