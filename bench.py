@@ -58,7 +58,7 @@ METRIC = "order-4 Sigma evals/s (samples x terms x frequencies, FP64), forward +
 # one, else the bench reports traffic as null.
 TRAFFIC = {"kernel": "tami_jit_fused (the diagram's specialised fused forward + adjoint)",
            "bytes_per_sample": (4.400048e9 + 5.369428e9) / 4194304,
-           "kernel_sha256": "26302a9b6702adf1ee4e31f770a5e863bb7577c29c169383b00d6e28be10e6e3",
+           "kernel_sha256": "bb6ea2188683d0b265dea352262ecbf0611fdc7359fb5e46b8187cd95a4f6576",
            "profile": "profiles/jit_kernels_order4_sigma.md"}
 
 

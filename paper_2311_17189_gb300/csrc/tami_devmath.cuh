@@ -164,7 +164,7 @@ __device__ __forceinline__ double rcp(double d) {
 // one, a sine within 6e-18 beside the last rounding (3.2 ulp at most); the sine within 3 pi/1024 of a
 // multiple of pi comes from sin_near, relatively accurate down to 0.  245 clocks of an SM quarter per
 // warp for a cosine, 1200 with an FP64 Taylor series to r^20; a line energy 355 against 1520, with its
-// gradients 690 against 2580 (order-5 forward, 2^23 samples, one frequency: 9.6 -> 5.6 ms; order-4
+// gradients 676 against 2580 (order-5 forward, 2^23 samples, one frequency: 9.6 -> 5.6 ms; order-4
 // forward + adjoint, 2^24 samples x 16 frequencies: 78.6 -> 71.9 ms).
 __device__ const __align__(16) unsigned long long kTrigTab[514] = {
   0x2000000000000000ull, 0x0000000000000000ull, 0x1fffd8858e8a924dull, 0x003243e1fcce00e2ull,
